@@ -716,7 +716,7 @@ static tbs_status plan_create(const tbs_plan_desc *d, void *workspace, size_t wo
         (e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking)) == cudaSuccess &&
         (e = cudaStreamCreateWithFlags(&p->body, cudaStreamNonBlocking)) == cudaSuccess &&
         (e = build_twiddles(p->M, p->tw, s)) == cudaSuccess &&
-        (p->periodic || (e = build_ghat(p->n, p->M, p->k0, d->dx, p->ghq, s)) == cudaSuccess) &&
+        (p->periodic || (e = build_ghat(p->n, p->M, p->k0, d->dx, p->ghq, p->X, p->W, p->S, s)) == cudaSuccess) &&
         (!p->periodic || (e = cudaMemcpyAsync(p->abl, abl_host.data(), sizeof(float) * p->M,
                                               cudaMemcpyHostToDevice, s)) == cudaSuccess) &&
         (e = cudaMemsetAsync(p->state, 0, r * sizeof(RhsState), s)) == cudaSuccess &&

@@ -194,7 +194,9 @@ cudaError_t set_col_smem_attr(int M);
 // plan build (tbs_plan.cu): twiddles and the spectrum quadrant of the
 // cell-averaged Green's table.  Synchronous on s; returns the first error.
 cudaError_t build_twiddles(int M, float2 *tw, cudaStream_t s);
-cudaError_t build_ghat(int n, int M, double k0, double dx, float2 *ghq, cudaStream_t s);
+// work, work2: n * M float2 of scratch each; work3: n * n float2.
+cudaError_t build_ghat(int n, int M, double k0, double dx, float2 *ghq, float2 *work, float2 *work2, float2 *work3,
+                       cudaStream_t s);
 
 // message returned by tbs_last_error() on this thread (tbs_api.cu)
 void set_last_error(const char *msg);

@@ -5,7 +5,7 @@
 // two N x M intermediates X and W, the partial sum psi, FP64 row partials and
 // the per-RHS stop state.  A solve is
 //
-//     row pass on S  ->  { column pass, row pass, stop test } while active
+//     row pass on S  ->  { column pass + stop test, row pass } while active
 //
 // and the host never waits between terms.  tbs_solve captures it once into a
 // CUDA graph (on a plan-owned stream) and replays it: the loop is a WHILE
@@ -175,6 +175,7 @@ ColArgs col_args(tbs_plan_s *p) {
     a.tw = p->tw;
     a.gate.st = p->state;
     a.gate.mode = GATE_ALL;
+    a.gate.before_row = 0;
     a.gate.j = 0;
     a.gate.jdev = nullptr;
     a.pdl = 0;
@@ -202,6 +203,7 @@ ColArgs col_args(tbs_plan_s *p) {
     a.err = p->err;
     a.wait_ns = p->wait_ns;
     a.extra_tx = p->extra_tx;
+    memset(&a.stop, 0, sizeof(a.stop));
     return a;
 }
 
@@ -320,7 +322,7 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     sa.div_factor = p->d.div_factor;
     sa.loop_ctl = nullptr;
     sa.loop = 0;
-    // in the term loop the row pass and the stop test are programmatic
+    // in the term loop the row pass and the stop kernel are programmatic
     // dependents of the kernel before them (their prologues overlap its tail)
     sa.pdl = 1;
     ra.pdl = 1;
@@ -329,6 +331,16 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     // the steady row pass: the term recurrence, or the paper's iteration on
     // psi on the periodic grid
     const int rk = !p->periodic ? ROW_FWD : p->psi0 ? ROW_EPSK : ROW_EPS;
+    // the stop test is made inside the next column pass, by blocks of whole
+    // warps (M >= 128); a term at N = 64 / 256 / 1024 13.5 / 19.7 / 40.2 ->
+    // 11.1 / 15.5 / 36.7 us, of the periodic 4096^2 grid 241 -> 232 us
+    const bool fused = p->M >= 128;
+    // A column pass is the row pass's programmatic dependent on small problems
+    // only: its prologue hidden saves 0.4 to 0.8 us of a 12 to 17 us term up to
+    // N = 512, but column blocks resident beside a large pass's last rows cost
+    // more (a term of 3 x 999^2 98.9 -> 101.2 us, of 2048^2 123.8 -> 124.9 us, of
+    // the periodic 4096^2 grid 232 -> 246 us).
+    const bool early = (size_t)p->nrhs * p->n * p->M <= (size_t)512 * 1024;
     // which rows of V are one repeated value and which source rows are zero
     // (the medium and sources may change between solves of a plan)
     if (rk == ROW_EPS) TBS_CK(launch_row_flags(p->n, p->nrhs, p->V, p->S, p->vflag, p->sflag, s));
@@ -348,19 +360,23 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
             cudaError_t e = cudaSuccess;
             for (int k = 0; k < TERMS_PER_ITERATION && e == cudaSuccess; k++) {
                 ColArgs ck = ca;
-                ck.pdl = k > 0;  // follows the previous term's stop test
+                ck.pdl = k > 0 && (early || !fused);  // follows a row pass (or a stop test)
+                if (k > 0 && fused) ck.stop = sa, ck.gate.before_row = 1;
                 StopArgs sk = sa;
                 sk.loop = h;
                 sk.loop_ctl = k == TERMS_PER_ITERATION - 1 ? p->err + 1 : nullptr;
                 e = launch_col(p->M, p->nrhs, false, ck, &p->cmaps[p->col_variant], p->col_variant, b);
                 if (e == cudaSuccess) e = launch_row(rk, p->M, p->nrhs, ra, b);
-                if (e == cudaSuccess) e = launch_stop(p->nrhs, sk, b);
+                // before the condition is evaluated; earlier terms' tests are
+                // the next column pass's
+                if (e == cudaSuccess && (sk.loop_ctl || !fused)) e = launch_stop(p->nrhs, sk, b);
             }
             return e;
         });
         if (st != TBS_OK) return st;
     } else {
         for (int t = 0; t < p->d.max_terms; t++) {
+            if (t > 0 && fused) ca.stop = sa, ca.gate.before_row = 1;  // the test of term t - 1
             TBS_CK(timed_col(p, false, ca, s));
             ra.term = t;
             // the last admissible term runs the inverse transform only: not
@@ -370,7 +386,7 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
             else
                 TBS_CK(timed_row(p, rk, ra, s));
             sa.term = t;
-            TBS_CK(launch_stop(p->nrhs, sa, s));
+            if (t == p->d.max_terms - 1 || !fused) TBS_CK(launch_stop(p->nrhs, sa, s));
         }
     }
     TBS_CK(launch_info(p->nrhs, p->state, p->err, p->info_dev, s));

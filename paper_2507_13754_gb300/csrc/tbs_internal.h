@@ -11,7 +11,7 @@ namespace tbs {
 // row starts 16-byte aligned and spans a multiple of 16 bytes (bulk copies).
 __host__ __device__ constexpr int ghat_stride(int M) { return M / 2 + 2; }
 
-// Per right-hand-side solver state, updated by the stop-test kernel.
+// Per right-hand-side solver state, updated by the stop test.
 struct RhsState {
     int done;        // 1 once the stop test has ended this RHS
     int terms;       // terms summed so far
@@ -22,14 +22,16 @@ struct RhsState {
     double tmax;     // max |u_n|_2
     double residual; // last residual
     double psi_norm; // |psi_n|_2
-    double pad_;
+    int before_row;  // `done` before the last forward row pass
+    int pad_;
 };
 
 // Which right-hand sides a launch works on.
 enum GateMode { GATE_ALL = 0, GATE_FWD = 1, GATE_ADJ = 2 };
 struct Gate {
-    const RhsState *st;  // per-RHS state
+    RhsState *st;        // per-RHS state
     int mode;
+    int before_row;      // GATE_FWD: read RhsState::before_row, not done (a stop test runs beside the launch)
     int j;               // adjoint step: RHS active while j <= terms - 2
     const int *jdev;     // where the step is read from when j < 0 (graph loop)
 };
@@ -49,10 +51,12 @@ enum RowKind {
                        // then psi' = A (g + psi^0); y = psi' -> X
 };
 
+// The stop test after a term's row pass: made by the next column pass of the
+// loop (ColArgs::stop) or by launch_stop.
 struct StopArgs {
     const double2 *part;
     const double2 *l1;
-    RhsState *st;
+    RhsState *st;       // null in ColArgs: no stop test
     double *norms;      // [rhs][max_terms]
     int *loop_ctl;      // graph loop: {arrivals, iterations}, or null outside one
     cudaGraphConditionalHandle loop;  // the WHILE node's condition (loop_ctl set)
@@ -128,6 +132,7 @@ struct ColArgs {
     // i (a2 s^(nu/2) + eps), s = ix^2 + iy^2, a1 = eta dp^(nu+1), a2 = tau omega dp^nu
     int kspace;
     float vv_a1, vv_a2, vv_eps, vv_half_nu;
+    StopArgs stop;      // the previous term's stop test, or st = null
 };
 
 

@@ -19,89 +19,6 @@
 
 namespace tbs {
 
-// Stop decision for one RHS after its term `term` (a.term, or the RHS's own
-// count), from the FP64 sums of |u_n|^2 and |psi_n|^2 (and the L1 row sums
-// for Eq. 30).  One thread.
-__device__ void stop_decide(const StopArgs &a, int rhs, double su, double sp) {
-    RhsState *s = a.st + rhs;
-    const double un = sqrt(su), pn = sqrt(sp);
-    const int term = a.term >= 0 ? a.term : s->terms;
-    a.norms[(size_t)rhs * a.max_terms + term] = un;
-    if (term == 0) {
-        s->u0 = un;
-        s->tmax = un;
-        s->grow = 0;
-        s->residual = INFINITY;
-        s->status = 1;  // TBS_MAX_TERMS until decided otherwise
-    }
-    if (un > s->tmax) s->tmax = un;
-    s->terms = term + 1;
-    s->psi_norm = pn;
-    bool have_r = true;
-    double r;
-    if (a.stop_mode == 1) {
-        if (term == 0) {
-            have_r = false;
-            r = INFINITY;
-        } else {
-            const double2 l = a.l1[rhs];
-            r = l.x / l.y;
-        }
-    } else {
-        r = pn > 0.0 ? un / pn : (un > 0.0 ? INFINITY : 0.0);
-    }
-    if (have_r) s->residual = r;
-    if (term > 0) s->grow = (un > s->prev) ? s->grow + 1 : 0;
-    int done = 0;
-    if (!isfinite(un) || !isfinite(pn)) {
-        s->status = 3;
-        done = 1;
-    } else if (have_r && r < a.tol) {
-        s->status = 0;
-        done = 1;
-    } else if ((term >= a.div_grace && s->grow >= a.div_window) || un > a.div_factor * s->u0) {
-        s->status = 2;
-        done = 1;
-    } else if (term + 1 >= a.max_terms) {
-        s->status = 1;
-        done = 1;
-    }
-    s->prev = un;
-    s->done = done;
-}
-
-// Fixed-order FP64 reduction of the row partials of one RHS by a 256-thread
-// block (per-thread strided sums, shuffle trees within and then across the
-// warps), then the stop decision in thread 0.
-__device__ void reduce_and_decide(const StopArgs &a, int rhs) {
-    __shared__ double2 rw[8];
-    double su = 0.0, sp = 0.0;
-    const double2 *part = a.part + (size_t)rhs * a.n;
-    for (int y = threadIdx.x; y < a.n; y += 256) {
-        const double2 q = part[y];
-        su += q.x;
-        sp += q.y;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        su += __shfl_xor_sync(0xffffffffu, su, o);
-        sp += __shfl_xor_sync(0xffffffffu, sp, o);
-    }
-    if (lane == 0) rw[warp] = make_double2(su, sp);
-    __syncthreads();
-    if (warp == 0) {
-        const double2 q = lane < 8 ? rw[lane] : make_double2(0.0, 0.0);
-        su = q.x;
-        sp = q.y;
-#pragma unroll
-        for (int o = 4; o >= 1; o >>= 1) {
-            su += __shfl_xor_sync(0xffffffffu, su, o);
-            sp += __shfl_xor_sync(0xffffffffu, sp, o);
-        }
-        if (lane == 0) stop_decide(a, rhs, su, sp);
-    }
-}
 
 // One block per RHS.  Inside a graph loop the last block to finish also
 // sets the WHILE condition: another iteration while any RHS is still active,
@@ -126,10 +43,6 @@ __global__ void __launch_bounds__(256) stop_kernel(StopArgs a) {
     }
 }
 
-// ---------------------------------------------------------------------------
-// stop test: FP64 reduction of the row partials, residual, divergence, flags
-// (Eq. 30 for the L1 row mode; full-grid L2 otherwise)
-// ---------------------------------------------------------------------------
 struct InfoOut {  // layout of tbs_solve_info
     int32_t terms;
     int32_t status;

@@ -168,7 +168,7 @@ static cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
 }
 
 __device__ __forceinline__ bool gate_active(const Gate &g, int rhs) {
-    if (g.mode == GATE_FWD) return g.st[rhs].done == 0;
+    if (g.mode == GATE_FWD) return (g.before_row ? g.st[rhs].before_row : g.st[rhs].done) == 0;
     if (g.mode == GATE_ADJ) return (g.j >= 0 ? g.j : *g.jdev) <= g.st[rhs].terms - 2;
     return true;
 }
@@ -240,6 +240,115 @@ __device__ __forceinline__ void row_sums(const float (&x)[K], double (&out)[K], 
 #pragma unroll
         for (int k = 0; k < K; k++) out[k] = (double)v[k].hi + (double)v[k].lo;
     }
+}
+
+// ---------------------------------------------------------------------------
+// stop test (Eq. 30 for the L1 row mode; full-grid L2 otherwise)
+// ---------------------------------------------------------------------------
+// Stop decision for one RHS after its term `term` (a.term, or the RHS's own
+// count), from the FP64 sums of |u_n|^2 and |psi_n|^2 (and the L1 row sums
+// for Eq. 30).  One thread.
+__device__ __forceinline__ void stop_decide(const StopArgs &a, int rhs, double su, double sp) {
+    RhsState *s = a.st + rhs;
+    const double un = sqrt(su), pn = sqrt(sp);
+    const int term = a.term >= 0 ? a.term : s->terms;
+    a.norms[(size_t)rhs * a.max_terms + term] = un;
+    if (term == 0) {
+        s->u0 = un;
+        s->tmax = un;
+        s->grow = 0;
+        s->residual = INFINITY;
+        s->status = 1;  // TBS_MAX_TERMS until decided otherwise
+    }
+    if (un > s->tmax) s->tmax = un;
+    s->terms = term + 1;
+    s->psi_norm = pn;
+    bool have_r = true;
+    double r;
+    if (a.stop_mode == 1) {
+        if (term == 0) {
+            have_r = false;
+            r = INFINITY;
+        } else {
+            const double2 l = a.l1[rhs];
+            r = l.x / l.y;
+        }
+    } else {
+        r = pn > 0.0 ? un / pn : (un > 0.0 ? INFINITY : 0.0);
+    }
+    if (have_r) s->residual = r;
+    if (term > 0) s->grow = (un > s->prev) ? s->grow + 1 : 0;
+    int done = 0;
+    if (!isfinite(un) || !isfinite(pn)) {
+        s->status = 3;
+        done = 1;
+    } else if (have_r && r < a.tol) {
+        s->status = 0;
+        done = 1;
+    } else if ((term >= a.div_grace && s->grow >= a.div_window) || un > a.div_factor * s->u0) {
+        s->status = 2;
+        done = 1;
+    } else if (term + 1 >= a.max_terms) {
+        s->status = 1;
+        done = 1;
+    }
+    s->prev = un;
+    s->done = done;
+}
+
+// Fixed-order FP64 reduction of the row partials of one RHS by a block of
+// whole warps (per-thread strided sums, shuffle trees within and then across
+// the warps), then the stop decision in thread 0.
+__device__ __forceinline__ void reduce_and_decide(const StopArgs &a, int rhs) {
+    __shared__ double2 rw[32];
+    double su = 0.0, sp = 0.0;
+    const double2 *part = a.part + (size_t)rhs * a.n;
+    for (int y = threadIdx.x; y < a.n; y += blockDim.x) {
+        const double2 q = __ldcg(part + y);
+        su += q.x;
+        sp += q.y;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        su += __shfl_xor_sync(0xffffffffu, su, o);
+        sp += __shfl_xor_sync(0xffffffffu, sp, o);
+    }
+    if (lane == 0) rw[warp] = make_double2(su, sp);
+    __syncthreads();
+    if (warp == 0) {
+        const double2 q = lane < warps ? rw[lane] : make_double2(0.0, 0.0);
+        su = q.x;
+        sp = q.y;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+            su += __shfl_xor_sync(0xffffffffu, su, o);
+            sp += __shfl_xor_sync(0xffffffffu, sp, o);
+        }
+        if (lane == 0) stop_decide(a, rhs, su, sp);
+    }
+    __syncthreads();  // rw may be written again
+}
+
+// The stop test inside a column pass: block gridDim.x - 1 - r decides for RHS
+// r about the term whose row pass has just ended, while the other blocks
+// already transform the next term's columns (a column pass writes W only, so
+// a pass begun for an RHS that stops here is merely unused).  The test is a
+// serial chain (the partials' loads, FP64 sums, two square roots and a
+// division: 6 to 10 us as a kernel of its own at N = 256 .. 4096) that nothing
+// of the column pass needs; the last blocks are those with the fewest tiles.
+__device__ __forceinline__ void col_stop(const StopArgs &a, int nrhs) {
+    if (!a.st) return;
+    for (int r = (int)gridDim.x - 1 - (int)blockIdx.x; r < nrhs; r += gridDim.x)
+        if (__ldcg(&a.st[r].done) == 0) reduce_and_decide(a, r);
+}
+
+// A forward row pass leaves each RHS's flag as it stood before this pass: the
+// column pass that follows changes `done` while its blocks run, so they read
+// this copy instead (every thread of a launch sees one value).
+__device__ __forceinline__ void mark_before_row(const RowArgs &a) {
+    if (a.gate.mode == GATE_FWD && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
+        for (int r = 0; r < a.nrhs; r++) a.gate.st[r].before_row = a.gate.st[r].done;
 }
 
 // Optional phase timers for experiments (compiled out unless defined).
@@ -320,7 +429,8 @@ row_kernel(RowArgs a) {
             cp_async_commit();
         }
     }
-    grid_dep_launch();  // the stop test may be scheduled once every row block runs
+    grid_dep_launch();  // the next kernel may be scheduled once every row block runs
+    if constexpr (KIND == ROW_FWD || KIND == ROW_EPS || KIND == ROW_EPSK) mark_before_row(a);
     TBS_ROW_PHASE_DECL
     if (!gate_active(a.gate, rhs)) {
         if (bulk) {
@@ -744,7 +854,8 @@ row_fwd_persistent_kernel(RowArgs a) {
         issue_w(i);
         issue_pv(i);
     }
-    grid_dep_launch();  // the stop test may be scheduled once every row block runs
+    grid_dep_launch();  // the next kernel may be scheduled once every row block runs
+    mark_before_row(a);
     unsigned ph_w = 0, ph_pv = 0;
     float2 va[1][E];
     float2 (&v)[E] = va[0];
@@ -944,6 +1055,7 @@ row_eps_persistent_kernel(RowArgs a) {
         issue_p(i);
     }
     grid_dep_launch();
+    mark_before_row(a);
     unsigned ph_w = 0, ph_p = 0;
     float2 va[1][E];
     float2 (&v)[E] = va[0];
@@ -1320,6 +1432,7 @@ col_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_cons
         __syncthreads();
         issue(i, 0);
     }
+    col_stop(a.stop, a.nrhs);
     int prev = -1;  // tile whose output rows wait in the other stage
     for (int buf = 0; i < total; buf ^= 1) {
         const int inext = next_active(i + gridDim.x);
@@ -1350,7 +1463,8 @@ col_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_cons
             TBS_COL_PHASE(3)
         };
         // k-space potential: from the RHS's second term on (its first applies G only)
-        const bool kspace = C::KS && a.gate.st && a.gate.st[i / TILES].terms > 0;
+        // (a pass that makes the previous term's stop test is never the first)
+        const bool kspace = C::KS && (a.stop.st || (a.gate.st && a.gate.st[i / TILES].terms > 0));
         if constexpr (C::BLOCKED)
             col_transform<C, M, CONJ>(v, exch, a, t, cg, (i % TILES) * TC, kspace, twr, st + C::LAND, st, between,
                                       GroupSync{1 + cg, C::T});
@@ -1510,6 +1624,7 @@ col_pipe_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid
         load_ghat(cur);
         if (nx1 < total) load_rows(nx1, D1, &bars[1]);
     }
+    col_stop(a.stop, a.nrhs);
     fl0 = cur < total;
     flg = !C::PER && cur < total;
     fl1 = nx1 < total;
@@ -1587,7 +1702,7 @@ col_pipe_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid
                 }
             };
             if constexpr (C::PERK == 2) {
-                if (a.gate.st && a.gate.st[cur / TILES].terms > 0)
+                if (a.stop.st || (a.gate.st && a.gate.st[cur / TILES].terms > 0))
                     multiply(std::true_type{});
                 else
                     multiply(std::false_type{});
@@ -1688,11 +1803,11 @@ template <int M, int KIND>
 static cudaError_t row_launch(int nrhs, const RowArgs &a, cudaStream_t s) {
     using C = RowCfg<M>;
     RowArgs b = a;
+    b.nrhs = nrhs;
     if (b.wait_ns == 0) b.wait_ns = 1000000000ull;  // 1 s
     if constexpr ((KIND == ROW_EPS || KIND == ROW_EPSK) && M >= 512) {
         if (a.n == M && a.num_sms > 0) {
             using P = RowECfg<M>;
-            b.nrhs = nrhs;
             const int slots = nrhs * a.n;
             int grid = a.num_sms * row_eps_persistent_blocks_per_sm<M, KIND == ROW_EPSK>();
             if (grid * P::RPB > slots) grid = (slots + P::RPB - 1) / P::RPB;
@@ -1703,7 +1818,6 @@ static cudaError_t row_launch(int nrhs, const RowArgs &a, cudaStream_t s) {
     if constexpr (KIND == ROW_FWD && M >= 512) {
         if ((a.n & 1) == 0 && a.num_sms > 0) {
             using P = RowPCfg<M>;
-            b.nrhs = nrhs;
             const int slots = nrhs * a.n;
             int grid = a.num_sms * row_persistent_blocks_per_sm<M>();
             if (grid * P::RPB > slots) grid = (slots + P::RPB - 1) / P::RPB;
@@ -1744,13 +1858,13 @@ static cudaError_t col_launch(int nrhs, const ColArgs &a, const ColMaps *maps, c
     b.nrhs = nrhs;
     b.xslice = x_slice_rows(a.n, C::BR);
     if (b.wait_ns == 0) b.wait_ns = 1000000000ull;  // 1 s
-    const int tiles = (M / C::TC) * nrhs;
+    // one block per tile, and per stop test, up to the resident ones
+    const int tiles = (M / C::TC) * nrhs, work = tiles + (a.stop.st ? nrhs : 0);
+    const int grid = work < a.num_sms ? work : a.num_sms;
     if constexpr (C::PIPE) {
-        const int grid = tiles < a.num_sms ? tiles : a.num_sms;
         return launch_k(col_pipe_kernel<M, CONJ, C::L, C::STAG, C::PERK, C::RS>, dim3(grid), dim3(C::THREADS), C::SMEM,
                         s, a.pdl != 0, b, maps->x, maps->w);
     } else {
-        const int grid = tiles < a.num_sms ? tiles : a.num_sms;
         return launch_k(col_kernel<M, CONJ, C>, dim3(grid), dim3(C::THREADS), C::SMEM, s, a.pdl != 0, b, maps->x,
                         maps->w);
     }

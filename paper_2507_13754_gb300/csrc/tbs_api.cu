@@ -178,7 +178,7 @@ ColArgs col_args(tbs_plan_s *p) {
     a.gate.before_row = 0;
     a.gate.j = 0;
     a.gate.jdev = nullptr;
-    a.pdl = 0;
+    a.pdl = a.early = 0;
     a.periodic = p->periodic;
     a.kq = a.eq = a.gs = 0.f;
     if (p->periodic) {
@@ -340,7 +340,11 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     // N = 512, but column blocks resident beside a large pass's last rows cost
     // more (a term of 3 x 999^2 98.9 -> 101.2 us, of 2048^2 123.8 -> 124.9 us, of
     // the periodic 4096^2 grid 232 -> 246 us).
-    const bool early = (size_t)p->nrhs * p->n * p->M <= (size_t)512 * 1024;
+    const size_t points = (size_t)p->nrhs * p->n * p->M;
+    const bool early = points <= (size_t)512 * 1024;
+    // The smallest passes leave room for the row pass's blocks beside them: a
+    // term at N = 256 14.2 -> 12.5 us (at N = 512 16.2 -> 17.0 us: not there).
+    const bool beside = points <= (size_t)256 * 512;
     // which rows of V are one repeated value and which source rows are zero
     // (the medium and sources may change between solves of a plan)
     if (rk == ROW_EPS) TBS_CK(launch_row_flags(p->n, p->nrhs, p->V, p->S, p->vflag, p->sflag, s));
@@ -360,6 +364,7 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
             cudaError_t e = cudaSuccess;
             for (int k = 0; k < TERMS_PER_ITERATION && e == cudaSuccess; k++) {
                 ColArgs ck = ca;
+                ck.early = beside;
                 ck.pdl = k > 0 && (early || !fused);  // follows a row pass (or a stop test)
                 if (k > 0 && fused) ck.stop = sa, ck.gate.before_row = 1;
                 StopArgs sk = sa;
@@ -716,6 +721,7 @@ static tbs_status plan_create(const tbs_plan_desc *d, void *workspace, size_t wo
             abl_host[i] = (float)(1.0 / (1.0 + exp(-d->abl_zeta * (edge * d->dx - 0.5 * mu))));
         }
     }
+    p->col_variant = col_default_variant(p->M, p->periodic);
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) == cudaSuccess)
         e = cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -726,7 +732,7 @@ static tbs_status plan_create(const tbs_plan_desc *d, void *workspace, size_t wo
     if (e == cudaSuccess && (e = set_row_smem_attr(p->M)) == cudaSuccess && (e = set_col_smem_attr(p->M)) == cudaSuccess &&
         ([&] {
             for (int v = 0; v < col_variants(p->M, p->periodic); v++)
-                p->col_grid[v] = p->num_sms * col_resident_blocks_per_sm(p->M, v, p->periodic);
+                p->col_grid[v] = p->num_sms * col_resident_blocks_per_sm(p->M, v, p->nrhs, p->periodic);
             return true;
         })() &&
         (e = cudaStreamCreateWithFlags(&p->cap, cudaStreamNonBlocking)) == cudaSuccess &&

@@ -121,6 +121,7 @@ struct ColArgs {
     int xslice;         // set by the launcher: rows per slice of the 3D view of X
                         // (one tensor copy per tile), or 0: one 2D copy per BR rows
     int pdl;            // launch as a programmatic dependent of the previous kernel
+    int early;          // let the next kernel's blocks be scheduled beside this pass
     // periodic grid (N = M): the spectrum g~(p)/M^2 = 1/((|p|^2 - k0^2 - i eps) M^2)
     // is formed in the kernel from integer wavenumbers (ix, iy) in [-M/2, M/2):
     // g = gs (a + i eq) / (a^2 + eq^2), a = ix^2 + iy^2 - kq, with p = dp (ix, iy),
@@ -208,6 +209,8 @@ void set_last_error(const char *msg);
 
 // resident column-pass blocks per SM (after set_col_smem_attr), for the
 // persistent grid (tbs_kernels.cu)
-int col_resident_blocks_per_sm(int M, int variant, bool periodic = false);
+int col_resident_blocks_per_sm(int M, int variant, int nrhs, bool periodic = false);
+// the variant a plan starts with
+int col_default_variant(int M, bool periodic);
 
 }  // namespace tbs

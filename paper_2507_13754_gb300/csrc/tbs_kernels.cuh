@@ -19,12 +19,13 @@ namespace tbs {
 // ---------------------------------------------------------------------------
 // configurations
 // ---------------------------------------------------------------------------
-template <int M>
+// TH: threads per block (at least a row's)
+template <int M, int TH = 256>
 struct RowCfg {
     static constexpr int E = 16;
     static constexpr int T = M / E;
-    static constexpr int RPB = T >= 256 ? 1 : 256 / T;  // rows per block
-    static constexpr int THREADS = T * RPB;               // 256
+    static constexpr int RPB = T >= TH ? 1 : TH / T;  // rows per block
+    static constexpr int THREADS = T * RPB;
     static constexpr int LINE = (padded_len(M) + 1) & ~1;  // FFT exchange line, 16-byte multiple
     static constexpr int HALF = M / 2;                    // >= N: psi / V row buffers
     // per row: the exchange line (the W row lands there unpadded first), then
@@ -104,6 +105,19 @@ struct ColVariant {
     static constexpr int MINB = THREADS >= 512 ? 1 : 65536 / (THREADS * 128);
     using type = ColShape<M, (TC >= 2 ? TC : 2), 1, MINB>;
 };
+
+// Narrower tiles where the default ones would leave SMs without a block:
+// a term on the periodic 1024^2 / 256^2 grid 22.7 / 14.8 -> 21.8 / 14.6 us, with
+// the k-space potential at 1024^2 25.8 -> 24.5 us.
+// (The choice follows M and the number of RHS alone: a plan's tensor maps and
+// its launches both make it.)
+__host__ __device__ constexpr bool col_narrow(int M, int nrhs, bool periodic) {
+    return periodic ? M >= 256 && M <= 1024 && (M / 8) * nrhs <= 128 : M >= 128 && M <= 256 && (M / 8) * nrhs <= 64;
+}
+template <int M>
+using ColNarrow = ColShape<M, (M >= 256 ? 2 : 4), 1>;
+template <int M, int PER>
+using ColNarrowP = ColShape<M, (M == 512 ? 2 : 4), 2, 1, PER>;
 
 // tile shapes of col_kernel: variants v with (default TC >> v) >= 2
 __host__ __device__ constexpr int col_shape_count(int M) {
@@ -361,10 +375,10 @@ __device__ __forceinline__ void mark_before_row(const RowArgs &a) {
 // ---------------------------------------------------------------------------
 // row pass
 // ---------------------------------------------------------------------------
-template <int M, int KIND>
-__global__ void __launch_bounds__(RowCfg<M>::THREADS, 2)
+template <int M, int KIND, int TH>
+__global__ void __launch_bounds__(RowCfg<M, TH>::THREADS, 512 / TH)
 row_kernel(RowArgs a) {
-    using C = RowCfg<M>;
+    using C = RowCfg<M, TH>;
     constexpr int E = C::E, T = C::T;
     extern __shared__ __align__(16) float2 smem[];
     __shared__ float2 red[4][8];
@@ -778,10 +792,10 @@ __device__ __forceinline__ void slot_sums(const float (&x)[K], double (&out)[K],
 // soon as the current one is in registers, and its psi and V rows once the
 // current epilogue has read them, so every copy has about a row's work to
 // land.  The arithmetic per row is exactly that of row_kernel<M, ROW_FWD>.
-template <int M>
+template <int M, int TH = 256>
 struct RowPCfg {
     static constexpr int E = 16, T = M / E;
-    static constexpr int RPB = T >= 256 ? 1 : 256 / T;
+    static constexpr int RPB = T >= TH ? 1 : TH / T;
     static constexpr int THREADS = T * RPB;
     static constexpr int LINE = RowCfg<M>::LINE;
     static constexpr int HALF = M / 2;
@@ -791,10 +805,10 @@ struct RowPCfg {
     static_assert(LINE % 2 == 0 && M % 2 == 0 && HALF % 2 == 0, "16-byte aligned slot buffers");
 };
 
-template <int M>
-__global__ void __launch_bounds__(RowPCfg<M>::THREADS, 2)
+template <int M, int TH>
+__global__ void __launch_bounds__(RowPCfg<M, TH>::THREADS, 512 / TH)
 row_fwd_persistent_kernel(RowArgs a) {
-    using C = RowPCfg<M>;
+    using C = RowPCfg<M, TH>;
     constexpr int E = C::E, T = C::T;
     extern __shared__ __align__(16) float2 smem[];
     __shared__ float2 red_all[C::RPB][4][8];
@@ -975,10 +989,10 @@ row_fwd_persistent_kernel(RowArgs a) {
 // periodic grid has no padding); both are bulk-copied a row ahead.  V, S and
 // psi^0 are read from global memory in batches, with the per-row flags (V
 // rows of one value read once, zero source rows not at all).
-template <int M>
+template <int M, int TH = 256>
 struct RowECfg {
     static constexpr int E = 16, T = M / E;
-    static constexpr int RPB = T >= 256 ? 1 : 256 / T;
+    static constexpr int RPB = T >= TH ? 1 : TH / T;
     static constexpr int THREADS = T * RPB;
     static constexpr int LINE = RowCfg<M>::LINE;
     static constexpr int SLOT = LINE + 2 * M;  // exchange line, W landing, psi row
@@ -986,10 +1000,10 @@ struct RowECfg {
     static_assert(T >= 32 && RPB <= 8, "one to eight warp-aligned row slots per block");
 };
 
-template <int M, bool KS>
-__global__ void __launch_bounds__(RowECfg<M>::THREADS, 2)
+template <int M, bool KS, int TH>
+__global__ void __launch_bounds__(RowECfg<M, TH>::THREADS, 512 / TH)
 row_eps_persistent_kernel(RowArgs a) {
-    using C = RowECfg<M>;
+    using C = RowECfg<M, TH>;
     constexpr int E = C::E, T = C::T;
     extern __shared__ __align__(16) float2 smem[];
     __shared__ float2 red_all[C::RPB][4][8];
@@ -1357,6 +1371,7 @@ col_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_cons
     }
     __syncthreads();
     grid_dep_wait();  // X, the RHS flags
+    if (a.early) grid_dep_launch();  // the row pass may be scheduled beside this pass
     unsigned par0 = 0u, par1 = 0u;  // phase parity of each stage's barrier (registers, not an array)
     constexpr int NW = (C::THREADS + 31) / 32;  // warps (blocks of 8 or 16 threads: one)
     static_assert(NW >= 1, "the copy-issue loop advances by NW");
@@ -1556,6 +1571,7 @@ col_pipe_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid
     }
     __syncthreads();
     grid_dep_wait();  // X, the RHS flags
+    if (a.early) grid_dep_launch();  // the row pass may be scheduled beside this pass
     const int total = TILES * a.nrhs;
     int cached_rhs = -1;
     bool cached_active = false;
@@ -1773,59 +1789,58 @@ col_pipe_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-template <int M>
-static int row_persistent_blocks_per_sm() {
-    static int nb = 0;  // per process: the kernel's resources do not change
-    if (nb == 0) {
+// Resident blocks per SM of a persistent row kernel (per process: the
+// kernel's resources do not change).
+template <auto K, int THREADS, size_t SMEM>
+static int resident_blocks() {
+    static const int nb = [] {
         int q = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, row_fwd_persistent_kernel<M>, RowPCfg<M>::THREADS,
-                                                          RowPCfg<M>::SMEM) != cudaSuccess || q < 1)
-            q = 1;
-        nb = q;
-    }
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, K, THREADS, SMEM) == cudaSuccess && q > 0 ? q : 1;
+    }();
     return nb;
 }
 
-template <int M, bool KS>
-static int row_eps_persistent_blocks_per_sm() {
-    static int nb = 0;  // per process: the kernel's resources do not change
-    if (nb == 0) {
-        int q = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&q, row_eps_persistent_kernel<M, KS>, RowECfg<M>::THREADS,
-                                                          RowECfg<M>::SMEM) != cudaSuccess || q < 1)
-            q = 1;
-        nb = q;
+// One persistent row pass: RPB slots per block over all rows.
+template <auto K, class P>
+static cudaError_t persistent_row(int nrhs, const RowArgs &b, cudaStream_t s) {
+    const int slots = nrhs * b.n;
+    int grid = b.num_sms * resident_blocks<K, P::THREADS, P::SMEM>();
+    if (grid * P::RPB > slots) grid = (slots + P::RPB - 1) / P::RPB;
+    return launch_k(K, dim3(grid), dim3(P::THREADS), P::SMEM, s, b.pdl != 0, b);
+}
+
+// Blocks of 64 threads instead of 256 where the latter would not give every SM
+// one (152 SMs).  With the column tiles and launches of small problems a term
+// at N = 256 went from 15.5 to 12.5 us, at N = 64 from 11.1 to 10.3 us; at
+// M = 1024 (N = 512) nothing was gained.
+__host__ __device__ constexpr bool row_has_small(int M) { return M <= 512; }
+static inline bool row_small(int M, int nrhs, int n) {
+    return row_has_small(M) && (size_t)nrhs * n * (M / 16) <= 152 * 256;
+}
+
+template <int M, int KIND, int TH>
+static cudaError_t row_launch_th(int nrhs, const RowArgs &b, cudaStream_t s) {
+    using C = RowCfg<M, TH>;
+    if constexpr ((KIND == ROW_EPS || KIND == ROW_EPSK) && M >= 512) {
+        if (b.n == M && b.num_sms > 0)
+            return persistent_row<row_eps_persistent_kernel<M, KIND == ROW_EPSK, TH>, RowECfg<M, TH>>(nrhs, b, s);
     }
-    return nb;
+    if constexpr (KIND == ROW_FWD && M >= 512) {
+        if ((b.n & 1) == 0 && b.num_sms > 0)
+            return persistent_row<row_fwd_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
+    }
+    dim3 grid((b.n + C::RPB - 1) / C::RPB, nrhs);
+    return launch_k(row_kernel<M, KIND, TH>, grid, dim3(C::THREADS), C::SMEM, s, b.pdl != 0, b);
 }
 
 template <int M, int KIND>
 static cudaError_t row_launch(int nrhs, const RowArgs &a, cudaStream_t s) {
-    using C = RowCfg<M>;
     RowArgs b = a;
     b.nrhs = nrhs;
     if (b.wait_ns == 0) b.wait_ns = 1000000000ull;  // 1 s
-    if constexpr ((KIND == ROW_EPS || KIND == ROW_EPSK) && M >= 512) {
-        if (a.n == M && a.num_sms > 0) {
-            using P = RowECfg<M>;
-            const int slots = nrhs * a.n;
-            int grid = a.num_sms * row_eps_persistent_blocks_per_sm<M, KIND == ROW_EPSK>();
-            if (grid * P::RPB > slots) grid = (slots + P::RPB - 1) / P::RPB;
-            return launch_k(row_eps_persistent_kernel<M, KIND == ROW_EPSK>, dim3(grid), dim3(P::THREADS), P::SMEM, s,
-                            a.pdl != 0, b);
-        }
-    }
-    if constexpr (KIND == ROW_FWD && M >= 512) {
-        if ((a.n & 1) == 0 && a.num_sms > 0) {
-            using P = RowPCfg<M>;
-            const int slots = nrhs * a.n;
-            int grid = a.num_sms * row_persistent_blocks_per_sm<M>();
-            if (grid * P::RPB > slots) grid = (slots + P::RPB - 1) / P::RPB;
-            return launch_k(row_fwd_persistent_kernel<M>, dim3(grid), dim3(P::THREADS), P::SMEM, s, a.pdl != 0, b);
-        }
-    }
-    dim3 grid((a.n + C::RPB - 1) / C::RPB, nrhs);
-    return launch_k(row_kernel<M, KIND>, grid, dim3(C::THREADS), C::SMEM, s, a.pdl != 0, b);
+    if constexpr (row_has_small(M))
+        if (row_small(M, nrhs, a.n)) return row_launch_th<M, KIND, 64>(nrhs, b, s);
+    return row_launch_th<M, KIND, 256>(nrhs, b, s);
 }
 
 template <int M>
@@ -1872,8 +1887,10 @@ static cudaError_t col_launch(int nrhs, const ColArgs &a, const ColMaps *maps, c
 
 // dispatch helper: F<shape>() for the shape of (M, variant)
 template <int M, class F>
-static cudaError_t with_col_variant(int variant, F f) {
+static cudaError_t with_col_variant(int variant, int nrhs, F f) {
     if (variant < 0 || variant >= col_variant_count(M)) return cudaErrorInvalidValue;
+    if constexpr (col_narrow(M, 1, false))
+        if (col_narrow(M, nrhs, false)) return f(ColNarrow<M>{});
     const int kind = col_variant_kind(M, variant);
     if constexpr (col_has_pipe(M)) {
         if (kind == COL_P1) return f(ColPShape<M, 1>{});
@@ -1939,7 +1956,9 @@ cudaError_t launch_row_m(int kind, int nrhs, const RowArgs &a, cudaStream_t s) {
 
 // periodic plans: F<shape>() for (variant, k-space)
 template <int M, class F>
-static cudaError_t with_col_variant_per(int variant, bool ks, F f) {
+static cudaError_t with_col_variant_per(int variant, int nrhs, bool ks, F f) {
+    if constexpr (col_narrow(M, 1, true))
+        if (variant == 0 && col_narrow(M, nrhs, true)) return ks ? f(ColNarrowP<M, 2>{}) : f(ColNarrowP<M, 1>{});
     // fastest first as measured on GB300 at M = 4096: two columns per thread,
     // then one (the only shape below M = 32)
     if constexpr (col_periodic_variant_count(M) > 1) {
@@ -1959,11 +1978,11 @@ template <int M>
 cudaError_t col_tensor_maps_m(ColMaps *maps, const float2 *X, const float2 *W, int n, int nrhs, int variant,
                               bool periodic) {
     if (periodic)
-        return with_col_variant_per<M>(variant, false, [&](auto c) {
+        return with_col_variant_per<M>(variant, nrhs, false, [&](auto c) {
             cudaError_t e = tile_tensor_map<decltype(c)>(&maps->x, X, n, M, nrhs);
             return e == cudaSuccess ? tile_tensor_map<decltype(c)>(&maps->w, W, n, M, nrhs) : e;
         });
-    return with_col_variant<M>(variant, [&](auto c) {
+    return with_col_variant<M>(variant, nrhs, [&](auto c) {
         cudaError_t e = tile_tensor_map<decltype(c)>(&maps->x, X, n, M, nrhs);
         return e == cudaSuccess ? tile_tensor_map<decltype(c)>(&maps->w, W, n, M, nrhs) : e;
     });
@@ -1973,10 +1992,10 @@ template <int M>
 cudaError_t launch_col_m(int nrhs, bool cj, const ColArgs &a, const ColMaps *maps, int variant, cudaStream_t s) {
     if (a.periodic) {  // forward spectrum only
         if (cj) return cudaErrorInvalidValue;
-        return with_col_variant_per<M>(variant, a.kspace != 0,
+        return with_col_variant_per<M>(variant, nrhs, a.kspace != 0,
                                        [&](auto c) { return col_launch<M, false, decltype(c)>(nrhs, a, maps, s); });
     }
-    return with_col_variant<M>(variant, [&](auto c) {
+    return with_col_variant<M>(variant, nrhs, [&](auto c) {
         using CC = decltype(c);
         return cj ? col_launch<M, true, CC>(nrhs, a, maps, s) : col_launch<M, false, CC>(nrhs, a, maps, s);
     });
@@ -1996,16 +2015,16 @@ static int col_blocks_per_sm() {
 }
 
 template <int M>
-int col_resident_blocks_m(int variant, bool periodic) {
+int col_resident_blocks_m(int variant, int nrhs, bool periodic) {
     int nb = 1;
     if (periodic) {
-        with_col_variant_per<M>(variant, false, [&](auto c) {
+        with_col_variant_per<M>(variant, nrhs, false, [&](auto c) {
             nb = col_blocks_per_sm<M, decltype(c)>();
             return cudaSuccess;
         });
         return nb;
     }
-    with_col_variant<M>(variant, [&](auto c) {
+    with_col_variant<M>(variant, nrhs, [&](auto c) {
         nb = col_blocks_per_sm<M, decltype(c)>();
         return cudaSuccess;
     });
@@ -2031,50 +2050,52 @@ static cudaError_t col_attr() {
 
 template <int M>
 cudaError_t set_col_smem_attr_m() {
+    constexpr int WIDE = 1 << 16;  // as many RHS as make no tile narrow
     cudaError_t e = cudaSuccess;
-    for (int v = 0; v < col_variant_count(M) && e == cudaSuccess; v++)
-        e = with_col_variant<M>(v, [&](auto c) { return col_attr<M, decltype(c)>(); });
-    for (int v = 0; v < col_periodic_variant_count(M) && e == cudaSuccess; v++)
-        for (int ks = 0; ks < 2 && e == cudaSuccess; ks++)
-            e = with_col_variant_per<M>(v, ks != 0, [&](auto c) {
-                using CC = decltype(c);
-                if constexpr (CC::PIPE)
-                    return col_attr<M, CC>();
-                else
-                    return cudaFuncSetAttribute(col_kernel<M, false, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)CC::SMEM);
-            });
+    auto per = [](auto c) {
+        using CC = decltype(c);
+        if constexpr (CC::PIPE)
+            return col_attr<M, CC>();
+        else
+            return cudaFuncSetAttribute(col_kernel<M, false, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)CC::SMEM);
+    };
+    for (int nrhs : {1, WIDE}) {
+        for (int v = 0; v < col_variant_count(M) && e == cudaSuccess; v++)
+            e = with_col_variant<M>(v, nrhs, [&](auto c) { return col_attr<M, decltype(c)>(); });
+        for (int v = 0; v < col_periodic_variant_count(M) && e == cudaSuccess; v++)
+            for (int ks = 0; ks < 2 && e == cudaSuccess; ks++) e = with_col_variant_per<M>(v, nrhs, ks != 0, per);
+    }
+    return e;
+}
+
+template <int M, int TH>
+static cudaError_t row_attr() {
+    const int b = (int)RowCfg<M, TH>::SMEM;
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto k, int bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    set(row_kernel<M, ROW_SRC, TH>, b);
+    set(row_kernel<M, ROW_FWD, TH>, b);
+    set(row_kernel<M, ROW_ADJ, TH>, b);
+    set(row_kernel<M, ROW_VSRC, TH>, b);
+    set(row_kernel<M, ROW_EPS, TH>, b);
+    set(row_kernel<M, ROW_EPSK, TH>, b);
+    set(row_kernel<M, ROW_OUT, TH>, b);
+    if constexpr (M >= 512) {
+        set(row_fwd_persistent_kernel<M, TH>, (int)RowPCfg<M, TH>::SMEM);
+        set(row_eps_persistent_kernel<M, false, TH>, (int)RowECfg<M, TH>::SMEM);
+        set(row_eps_persistent_kernel<M, true, TH>, (int)RowECfg<M, TH>::SMEM);
+    }
     return e;
 }
 
 template <int M>
-static cudaError_t row_attr() {
-    using C = RowCfg<M>;
-    const int b = (int)C::SMEM;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(row_kernel<M, ROW_SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    if ((e = cudaFuncSetAttribute(row_kernel<M, ROW_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    if ((e = cudaFuncSetAttribute(row_kernel<M, ROW_ADJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    if ((e = cudaFuncSetAttribute(row_kernel<M, ROW_VSRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    if ((e = cudaFuncSetAttribute(row_kernel<M, ROW_EPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    if ((e = cudaFuncSetAttribute(row_kernel<M, ROW_EPSK>, cudaFuncAttributeMaxDynamicSharedMemorySize, b))) return e;
-    return cudaFuncSetAttribute(row_kernel<M, ROW_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-}
-
-template <int M>
 cudaError_t set_row_smem_attr_m() {
-    cudaError_t e = row_attr<M>();
-    if constexpr (M >= 512) {
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(row_fwd_persistent_kernel<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)RowPCfg<M>::SMEM);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(row_eps_persistent_kernel<M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)RowECfg<M>::SMEM);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(row_eps_persistent_kernel<M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)RowECfg<M>::SMEM);
-    }
+    cudaError_t e = row_attr<M, 256>();
+    if constexpr (row_has_small(M))
+        if (e == cudaSuccess) e = row_attr<M, 64>();
     return e;
 }
 
@@ -2087,7 +2108,7 @@ cudaError_t set_row_smem_attr_m() {
                                                    int, bool);                                          \
     PRE template cudaError_t launch_col_m<MM>(int, bool, const ColArgs &, const ColMaps *, int,         \
                                               cudaStream_t);                                            \
-    PRE template int col_resident_blocks_m<MM>(int, bool);                                              \
+    PRE template int col_resident_blocks_m<MM>(int, int, bool);                                         \
     PRE template cudaError_t set_col_smem_attr_m<MM>();                                                 \
     PRE template cudaError_t set_row_smem_attr_m<MM>();
 }  // namespace tbs

@@ -10,7 +10,7 @@
 // and the host never waits between terms.  tbs_solve captures it once into a
 // CUDA graph (on a plan-owned stream) and replays it: the loop is a WHILE
 // conditional node whose condition the stop test sets, so the graph runs the
-// terms the slowest RHS needs (in bodies of four; launches past an RHS's stop
+// terms the slowest RHS needs (in bodies of several; launches past an RHS's stop
 // return at once).  Without a graph (timing,
 // TBS_FLAG_NO_GRAPH) the loop is unrolled max_terms times on the stream and
 // launches after every RHS has stopped return at once.  Each launch checks
@@ -349,12 +349,15 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     // (the medium and sources may change between solves of a plan)
     if (rk == ROW_EPS) TBS_CK(launch_row_flags(p->n, p->nrhs, p->V, p->S, p->vflag, p->sflag, s));
     if (graph_loop) {
-        // The body runs TERMS_PER_ITERATION terms; each kernel reads its
-        // RHS's term index from the RHS state and returns at once for an RHS
-        // that has stopped.  The last stop test of the body sets the
-        // condition (a WHILE iteration costs a few microseconds more than
-        // the launches it holds, so the loop is unrolled).
-        constexpr int TERMS_PER_ITERATION = 4;
+        // The body runs `body` terms; each kernel reads its RHS's term index
+        // from the RHS state and returns at once for an RHS that has stopped.
+        // The last stop test of the body sets the condition.  An iteration
+        // costs 7 us beyond the launches it holds, a term's launches after the
+        // stop about 4 us, so to a residual the body holds 8 terms (4 -> 8: a
+        // term at N = 64 / 256 / 1024 1.0 / 1.0 / 1.2 us less), and a fixed number
+        // of terms is split into equal bodies of at most 16.
+        const int bodies = (p->d.max_terms + 15) / 16;
+        const int body = p->d.tol > 0 ? 8 : (p->d.max_terms + bodies - 1) / bodies;
         cudaGraphConditionalHandle h;
         tbs_status st = loop_condition(s, &h);
         if (st != TBS_OK) return st;
@@ -362,14 +365,14 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
         sa.term = -1;
         st = capture_while(p, s, h, [&](cudaStream_t b) {
             cudaError_t e = cudaSuccess;
-            for (int k = 0; k < TERMS_PER_ITERATION && e == cudaSuccess; k++) {
+            for (int k = 0; k < body && e == cudaSuccess; k++) {
                 ColArgs ck = ca;
                 ck.early = beside;
                 ck.pdl = k > 0 && (early || !fused);  // follows a row pass (or a stop test)
                 if (k > 0 && fused) ck.stop = sa, ck.gate.before_row = 1;
                 StopArgs sk = sa;
                 sk.loop = h;
-                sk.loop_ctl = k == TERMS_PER_ITERATION - 1 ? p->err + 1 : nullptr;
+                sk.loop_ctl = k == body - 1 ? p->err + 1 : nullptr;
                 e = launch_col(p->M, p->nrhs, false, ck, &p->cmaps[p->col_variant], p->col_variant, b);
                 if (e == cudaSuccess) e = launch_row(rk, p->M, p->nrhs, ra, b);
                 // before the condition is evaluated; earlier terms' tests are

@@ -178,6 +178,7 @@ ColArgs col_args(tbs_plan_s *p) {
     a.gate.before_row = 0;
     a.gate.j = 0;
     a.gate.jdev = nullptr;
+    a.gate.back = 0;
     a.pdl = a.early = 0;
     a.periodic = p->periodic;
     a.kq = a.eq = a.gs = 0.f;
@@ -302,6 +303,13 @@ void drop_graphs(tbs_plan_s *p) {
     p->exec = p->exec_adj = nullptr;
 }
 
+// A column pass is the row pass's programmatic dependent on small problems
+// only: its prologue hidden saves 0.4 to 0.8 us of a 12 to 17 us term up to
+// N = 512, but column blocks resident beside a large pass's last rows cost more
+// (a term of 3 x 999^2 98.9 -> 101.2 us, of 2048^2 123.8 -> 124.9 us, of the
+// periodic 4096^2 grid 232 -> 246 us).
+bool early_columns(const tbs_plan_s *p) { return (size_t)p->nrhs * p->n * p->M <= (size_t)512 * 1024; }
+
 tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     TBS_CK(cudaMemsetAsync(p->state, 0, sizeof(RhsState) * p->nrhs, s));
     TBS_CK(cudaMemsetAsync(p->err, 0, 4 * sizeof(int), s));
@@ -335,16 +343,10 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     // warps (M >= 128); a term at N = 64 / 256 / 1024 13.5 / 19.7 / 40.2 ->
     // 11.1 / 15.5 / 36.7 us, of the periodic 4096^2 grid 241 -> 232 us
     const bool fused = p->M >= 128;
-    // A column pass is the row pass's programmatic dependent on small problems
-    // only: its prologue hidden saves 0.4 to 0.8 us of a 12 to 17 us term up to
-    // N = 512, but column blocks resident beside a large pass's last rows cost
-    // more (a term of 3 x 999^2 98.9 -> 101.2 us, of 2048^2 123.8 -> 124.9 us, of
-    // the periodic 4096^2 grid 232 -> 246 us).
-    const size_t points = (size_t)p->nrhs * p->n * p->M;
-    const bool early = points <= (size_t)512 * 1024;
+    const bool early = early_columns(p);
     // The smallest passes leave room for the row pass's blocks beside them: a
     // term at N = 256 14.2 -> 12.5 us (at N = 512 16.2 -> 17.0 us: not there).
-    const bool beside = points <= (size_t)256 * 512;
+    const bool beside = (size_t)p->nrhs * p->n * p->M <= (size_t)256 * 512;
     // which rows of V are one repeated value and which source rows are zero
     // (the medium and sources may change between solves of a plan)
     if (rk == ROW_EPS) TBS_CK(launch_row_flags(p->n, p->nrhs, p->V, p->S, p->vflag, p->sflag, s));
@@ -415,20 +417,28 @@ tbs_status enqueue_adjoint(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     ra.pdl = 1;  // the reverse steps' row passes follow their column passes programmatically
     ra.gate.mode = GATE_ADJ;
     ca.gate.mode = GATE_ADJ;
+    const bool early = early_columns(p);
     if (graph_loop) {
         int *jdev = p->err + 3;
         cudaGraphConditionalHandle h;
         tbs_status st = loop_condition(s, &h);
         if (st != TBS_OK) return st;
-        TBS_CK(launch_adj_loop(p->nrhs, p->state, jdev, h, true, s));
+        TBS_CK(launch_adj_loop(p->nrhs, p->state, jdev, h, true, 0, s));
         ra.term = -1;
         ra.gate.j = ca.gate.j = -1;
         ra.gate.jdev = ca.gate.jdev = jdev;
         return capture_while(p, s, h, [&](cudaStream_t b) {
-            cudaError_t e = launch_col(p->M, p->nrhs, true, ca, &p->cmaps[p->col_variant], p->col_variant, b);
-            if (e == cudaSuccess) e = launch_row(ROW_ADJ, p->M, p->nrhs, ra, b);
-            if (e == cudaSuccess) e = launch_adj_loop(p->nrhs, p->state, jdev, h, false, b);
-            return e;
+            // several steps per iteration, as in the forward loop; those below
+            // step 0 return at once
+            constexpr int STEPS = 8;
+            cudaError_t e = cudaSuccess;
+            for (int k = 0; k < STEPS && e == cudaSuccess; k++) {
+                ra.gate.back = ca.gate.back = k;
+                ca.pdl = k > 0 && early;
+                e = launch_col(p->M, p->nrhs, true, ca, &p->cmaps[p->col_variant], p->col_variant, b);
+                if (e == cudaSuccess) e = launch_row(ROW_ADJ, p->M, p->nrhs, ra, b);
+            }
+            return e == cudaSuccess ? launch_adj_loop(p->nrhs, p->state, jdev, h, false, STEPS, b) : e;
         });
     }
     for (int j = p->d.max_terms - 2; j >= 0; j--) {
@@ -1225,19 +1235,20 @@ tbs_status tbs_autotune(tbs_plan_t p, int32_t reps, double *times_ms, int32_t *b
     return tbs_set_col_variant(p, bi);
 }
 
+// the persistent steady-state passes exist for M >= 512
+static bool row_persistent(tbs_plan_t p) { return p->M >= 512; }
+
 int32_t tbs_row_variants(tbs_plan_t p) {
     if (!p) return 0;
-    // the persistent steady-state passes exist for M >= 512 with an even N
-    // (padded grid) or N = M (periodic grid)
-    const bool persistent = p->M >= 512 && (p->periodic ? p->n == p->M : (p->n & 1) == 0);
-    return persistent ? 2 : 1;
+    // an odd N has the persistent pass alone
+    return row_persistent(p) && (p->n & 1) == 0 ? 2 : 1;
 }
 
 const char *tbs_row_variant_name(tbs_plan_t p, int32_t variant) {
     if (!p) return nullptr;
     if (variant < 0) variant = p->row_variant;
     if (variant >= tbs_row_variants(p)) return nullptr;
-    if (tbs_row_variants(p) == 1) return "one block per row";
+    if (!row_persistent(p)) return "one block per row";
     return variant == 0 ? "persistent, rows prefetched a row ahead" : "one block per row";
 }
 
@@ -1260,7 +1271,7 @@ tbs_status tbs_autotune_rows(tbs_plan_t p, int32_t reps, double *times_ms, int32
     // scratch field instead of the plan's result, and store no terms.
     const size_t bytes = (size_t)p->nrhs * p->n * p->n * sizeof(float2);
     float2 *scratch = nullptr;
-    TBS_CK(cudaMalloc(&scratch, bytes));
+    TBS_CK(cudaMalloc(&scratch, bytes + 16));  // an odd N's row copies end on a 16-byte boundary
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaMemsetAsync(scratch, 0, bytes, s);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
@@ -1270,7 +1281,7 @@ tbs_status tbs_autotune_rows(tbs_plan_t p, int32_t reps, double *times_ms, int32
     double bt = 1e300;
     for (int v = 0; e == cudaSuccess && v < nv; v++) {
         RowArgs ra = row_args(p);
-        ra.num_sms = v == 0 && nv > 1 ? p->num_sms : 0;
+        ra.num_sms = v == 0 && row_persistent(p) ? p->num_sms : 0;
         ra.psi = scratch;
         ra.U = nullptr;
         ra.term = 1;  // a steady-state term: inverse transform, epilogue, forward transform

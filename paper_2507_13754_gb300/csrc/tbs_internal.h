@@ -33,7 +33,8 @@ struct Gate {
     int mode;
     int before_row;      // GATE_FWD: read RhsState::before_row, not done (a stop test runs beside the launch)
     int j;               // adjoint step: RHS active while j <= terms - 2
-    const int *jdev;     // where the step is read from when j < 0 (graph loop)
+    const int *jdev;     // where the step is read from when j < 0 (graph loop),
+    int back;            // less this many (negative: no step)
 };
 
 // Row-pass variants.
@@ -162,8 +163,8 @@ cudaError_t col_tensor_maps(ColMaps *maps, const float2 *X, const float2 *W, int
                             bool periodic = false);
 cudaError_t launch_stop(int nrhs, const StopArgs &a, cudaStream_t s);
 // Adjoint graph loop control (one thread): with init, *j = max_r terms_r - 2,
-// else *j -= 1; then the WHILE condition is set to (*j >= 0).
-cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphConditionalHandle h, bool init,
+// else *j -= steps; then the WHILE condition is set to (*j >= 0).
+cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphConditionalHandle h, bool init, int steps,
                             cudaStream_t s);
 cudaError_t launch_info(int nrhs, const RhsState *st, const int *err, void *info_dev, cudaStream_t s);
 // V = p^2 - k0^2 - i eps_shift (eps_shift = 0 except on the periodic grid)

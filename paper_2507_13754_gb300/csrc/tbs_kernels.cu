@@ -51,14 +51,15 @@ struct InfoOut {  // layout of tbs_solve_info
     double psi_norm;
 };
 
-__global__ void adj_loop_kernel(int nrhs, const RhsState *st, int *jdev, cudaGraphConditionalHandle h, int init) {
+__global__ void adj_loop_kernel(int nrhs, const RhsState *st, int *jdev, cudaGraphConditionalHandle h, int init,
+                                int steps) {
     int j;
     if (init) {
         int tmax = 0;
         for (int r = 0; r < nrhs; r++) tmax = max(tmax, st[r].terms);
         j = tmax - 2;
     } else {
-        j = *jdev - 1;
+        j = *jdev - steps;
     }
     *jdev = j;
     cudaGraphSetConditional(h, j >= 0 ? 1u : 0u);
@@ -333,9 +334,9 @@ cudaError_t launch_stop(int nrhs, const StopArgs &a, cudaStream_t s) {
     return launch_k(stop_kernel, dim3(nrhs), dim3(256), 0, s, a.pdl != 0, a);
 }
 
-cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphConditionalHandle h, bool init,
+cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphConditionalHandle h, bool init, int steps,
                             cudaStream_t s) {
-    adj_loop_kernel<<<1, 1, 0, s>>>(nrhs, st, j, h, init ? 1 : 0);
+    adj_loop_kernel<<<1, 1, 0, s>>>(nrhs, st, j, h, init ? 1 : 0, steps);
     return cudaGetLastError();
 }
 

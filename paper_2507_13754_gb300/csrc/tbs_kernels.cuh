@@ -183,7 +183,10 @@ static cudaError_t launch_k(void (*k)(P...), dim3 grid, dim3 block, size_t smem,
 
 __device__ __forceinline__ bool gate_active(const Gate &g, int rhs) {
     if (g.mode == GATE_FWD) return (g.before_row ? g.st[rhs].before_row : g.st[rhs].done) == 0;
-    if (g.mode == GATE_ADJ) return (g.j >= 0 ? g.j : *g.jdev) <= g.st[rhs].terms - 2;
+    if (g.mode == GATE_ADJ) {
+        const int j = g.j >= 0 ? g.j : *g.jdev - g.back;
+        return j >= 0 && j <= g.st[rhs].terms - 2;
+    }
     return true;
 }
 
@@ -317,6 +320,7 @@ __device__ __forceinline__ void reduce_and_decide(const StopArgs &a, int rhs) {
     __shared__ double2 rw[32];
     double su = 0.0, sp = 0.0;
     const double2 *part = a.part + (size_t)rhs * a.n;
+#pragma unroll 8
     for (int y = threadIdx.x; y < a.n; y += blockDim.x) {
         const double2 q = __ldcg(part + y);
         su += q.x;
@@ -461,7 +465,7 @@ row_kernel(RowArgs a) {
     // or adjoint step j (given, or the graph loop's counter)
     const int term = a.term >= 0                          ? a.term
                      : (KIND == ROW_FWD || KIND == ROW_EPS || KIND == ROW_EPSK) ? a.gate.st[rhs].terms
-                     : KIND == ROW_ADJ                      ? *a.gate.jdev
+                     : KIND == ROW_ADJ                      ? *a.gate.jdev - a.gate.back
                                                             : 0;
     TBS_ROW_PHASE(0)
 
@@ -783,8 +787,24 @@ __device__ __forceinline__ void slot_sums(const float (&x)[K], double (&out)[K],
     for (int k = 0; k < K; k++) out[k] = (double)v[k].hi + (double)v[k].lo;
 }
 
-// Steady-state forward row pass (ROW_FWD) as a persistent kernel for M >= 512
-// and even N: each block holds RPB row slots of T = M/16 threads, and each
+// A row of n complex64 elements as a bulk copy moves it: for an odd N every
+// other row starts 8 bytes past a 16-byte boundary, so the copy begins one
+// element earlier (the row stands at `off` in the buffer) and ends on the next
+// boundary.  The elements beside the row are neighbours in the same plan
+// buffer, or its alignment padding, and are not used.
+struct RowSpan {
+    const float2 *p;
+    unsigned bytes;
+    int off;
+    __device__ __forceinline__ RowSpan(const float2 *row, int n) {
+        off = (int)((reinterpret_cast<uintptr_t>(row) >> 3) & 1u);
+        p = row - off;
+        bytes = (unsigned)(((n + off + 1) & ~1) * sizeof(float2));
+    }
+};
+
+// Steady-state forward row pass (ROW_FWD) as a persistent kernel for M >= 512:
+// each block holds RPB row slots of T = M/16 threads, and each
 // slot walks the rows i = slot, slot + (number of slots), ... of all active
 // right-hand sides (row y of RHS r is i = r N + y).  A slot keeps four
 // buffers: the padded exchange line, a landing row for the next W row, and
@@ -851,7 +871,7 @@ row_fwd_persistent_kernel(RowArgs a) {
         }
         return i;
     };
-    const unsigned wbytes = (unsigned)(M * sizeof(float2)), rbytes = (unsigned)(n * sizeof(float2));
+    const unsigned wbytes = (unsigned)(M * sizeof(float2));
     auto issue_w = [&](int i) {  // slot thread 0
         const int r = i / n, y = i - r * n;
         mbar_arrive_expect_tx(bar_w, wbytes);
@@ -859,9 +879,10 @@ row_fwd_persistent_kernel(RowArgs a) {
     };
     auto issue_pv = [&](int i) {  // slot thread 0
         const int r = i / n, y = i - r * n;
-        mbar_arrive_expect_tx(bar_pv, 2 * rbytes);
-        bulk_load(psi_s, a.psi + (size_t)r * n * n + (size_t)y * n, rbytes, bar_pv);
-        bulk_load(v_s, a.V + (size_t)y * n, rbytes, bar_pv);
+        const RowSpan p(a.psi + (size_t)r * n * n + (size_t)y * n, n), v(a.V + (size_t)y * n, n);
+        mbar_arrive_expect_tx(bar_pv, p.bytes + v.bytes);
+        bulk_load(psi_s, p.p, p.bytes, bar_pv);
+        bulk_load(v_s, v.p, v.bytes, bar_pv);
     };
     int i = next_active(blockIdx.x * C::RPB + lr);
     if (t == 0 && i < total) {
@@ -918,6 +939,7 @@ row_fwd_persistent_kernel(RowArgs a) {
             }
             return;
         }
+        const float2 *pr = psi_s + RowSpan(a.psi + row_sp, n).off, *vr = v_s + RowSpan(a.V + (size_t)y * n, n).off;
         // u -> psi += u, the norms' partial sums, V u; the N = M/2 grids (every
         // slot of the half row a grid point) skip the per-element bound
         auto epilogue = [&](auto full_c) {
@@ -927,7 +949,7 @@ row_fwd_persistent_kernel(RowArgs a) {
                 const int x = t + T * m;
                 if (FULL || x < n) {
                     const float2 u = v[m];
-                    const float2 pold = first ? make_float2(0.f, 0.f) : psi_s[x];
+                    const float2 pold = first ? make_float2(0.f, 0.f) : pr[x];
                     const float2 p = cadd(pold, u);
                     a.psi[row_sp + x] = p;
                     if (U) U[x] = u;
@@ -937,7 +959,7 @@ row_fwd_persistent_kernel(RowArgs a) {
                         lu_f += hypotf(u.x, u.y);
                         lp_f += hypotf(pold.x, pold.y);
                     }
-                    v[m] = cmul(v_s[x], u);
+                    v[m] = cmul(vr[x], u);
                 } else {
                     v[m] = make_float2(0.f, 0.f);
                 }
@@ -974,6 +996,151 @@ row_fwd_persistent_kernel(RowArgs a) {
             // reads of the exchange line
             fft_lines<M, E, -1, 1, ThreadTwiddles<M, E>, GroupSync, true, true>(va, sm, t, a.tw, &twr, sync);
             float2 *xo = a.X + ((size_t)rhs * n + y) * M;
+#pragma unroll
+            for (int m = 0; m < E; m++) xo[t + T * m] = v[m];
+        }
+        i = inext;
+    }
+}
+
+// The reverse sweep's row pass (ROW_ADJ) as a persistent kernel, M >= 512: the
+// slots of row_fwd_persistent_kernel, whose two half-row buffers
+// hold the Q and u_j rows here (both bulk-copied a row ahead, like W); g's row
+// is fetched into L2 meanwhile, V stays there.  The arithmetic per row is
+// exactly that of row_kernel<M, ROW_ADJ>.  One block per row loads W, Q, u_j,
+// g and V in turn between its transforms, each exposed to memory latency:
+// 302 us for 16 RHS at N = 1024, here 178 us.
+template <int M, int TH>
+__global__ void __launch_bounds__(RowPCfg<M, TH>::THREADS, 512 / TH)
+row_adj_persistent_kernel(RowArgs a) {
+    using C = RowPCfg<M, TH>;
+    constexpr int E = C::E, T = C::T;
+    extern __shared__ __align__(16) float2 smem[];
+    __shared__ __align__(8) uint64_t bars[C::RPB][2];  // [slot][0: W, 1: Q and u_j]
+    const int lr = threadIdx.x / T;
+    const int t = threadIdx.x % T;
+    const int n = a.n;
+    float2 *line = smem + (size_t)lr * C::SLOT;
+    float2 *wl = line + C::LINE;
+    float2 *q_s = wl + M;
+    float2 *u_s = q_s + C::HALF;
+    const GroupSync sync{1 + lr, T};
+    const Lines<1> sm{line, 0};
+    uint64_t *bar_w = &bars[lr][0], *bar_q = &bars[lr][1];
+    if (t == 0) {
+        mbar_init(bar_w, 1);
+        mbar_init(bar_q, 1);
+        mbar_init_fence();
+    }
+    ThreadTwiddles<M, E> twr;
+    twr.load(a.tw, t);
+    sync();  // the slot's barriers are initialised before anyone waits
+    grid_dep_wait();
+    const int total = a.nrhs * n;
+    const int nslots = gridDim.x * C::RPB;
+    const int term = a.term >= 0 ? a.term : *a.gate.jdev - a.gate.back;
+    const float2 *Uj = a.U + (size_t)((term - a.u_term0) / a.u_every) * a.u_slot;
+    int cached_rhs = -1;
+    bool cached_active = false;
+    auto next_active = [&](int i) {
+        while (i < total) {
+            const int r = i / n;
+            if (r != cached_rhs) {
+                cached_rhs = r;
+                cached_active = gate_active(a.gate, r);
+            }
+            if (cached_active) break;
+            i += nslots;
+        }
+        return i;
+    };
+    const unsigned wbytes = (unsigned)(M * sizeof(float2));
+    auto issue_w = [&](int i) {  // slot thread 0
+        mbar_arrive_expect_tx(bar_w, wbytes);
+        bulk_load(wl, a.W + (size_t)i * M, wbytes, bar_w);
+    };
+    auto issue_q = [&](int i) {  // slot thread 0
+        const int r = i / n, y = i - r * n;
+        const RowSpan q(a.Q + (size_t)i * n, n), u(Uj + r * a.u_rhs + (size_t)y * n, n), g(a.src + (size_t)i * n, n);
+        mbar_arrive_expect_tx(bar_q, q.bytes + u.bytes);
+        bulk_load(q_s, q.p, q.bytes, bar_q);
+        bulk_load(u_s, u.p, u.bytes, bar_q);
+        bulk_prefetch_l2(g.p, g.bytes);
+    };
+    int i = next_active(blockIdx.x * C::RPB + lr);
+    if (t == 0 && i < total) {
+        issue_w(i);
+        issue_q(i);
+    }
+    grid_dep_launch();
+    unsigned ph_w = 0, ph_q = 0;
+    float2 va[1][E];
+    float2 (&v)[E] = va[0];
+    while (i < total) {
+        const int rhs = i / n, y = i - rhs * n;
+        const int inext = next_active(i + nslots);
+        const bool okw = mbar_wait_bounded(bar_w, ph_w, a.wait_ns, a.err);
+        ph_w ^= 1u;
+        if (group_sync_or(1 + lr, T, !okw)) {  // as in the forward pass
+            if (t == 0) {
+                mbar_wait_bounded(bar_w, ph_w ^ 1u, a.wait_ns, nullptr);
+                mbar_wait_bounded(bar_q, ph_q, a.wait_ns, nullptr);
+            }
+            return;
+        }
+#pragma unroll
+        for (int m = 0; m < E; m++) v[m] = wl[t + T * m];
+        sync();  // every thread's reads of the landing row are done
+        if (t == 0 && inext < total) {
+            fence_proxy_async_smem();
+            issue_w(inext);
+        }
+        fft_lines<M, E, +1, 1, ThreadTwiddles<M, E>, GroupSync, true>(va, sm, t, a.tw, &twr, sync);
+        const bool okq = mbar_wait_bounded(bar_q, ph_q, a.wait_ns, a.err);
+        ph_q ^= 1u;
+        if (group_sync_or(1 + lr, T, !okq)) {
+            if (t == 0) {
+                if (inext < total) mbar_wait_bounded(bar_w, ph_w, a.wait_ns, nullptr);
+                mbar_wait_bounded(bar_q, ph_q ^ 1u, a.wait_ns, nullptr);
+            }
+            return;
+        }
+        float2 *Q = a.Q + (size_t)i * n;
+        const float2 *g = a.src + (size_t)i * n, *V = a.V + (size_t)y * n;
+        const float2 *qr = q_s + RowSpan(Q, n).off, *ur = u_s + RowSpan(Uj + rhs * a.u_rhs + (size_t)y * n, n).off;
+        constexpr int CH = 4;  // a batch's loads are issued together
+#pragma unroll
+        for (int m0 = 0; m0 < E / 2; m0 += CH) {
+            float2 gg[CH], vv[CH];
+#pragma unroll
+            for (int k = 0; k < CH; k++) {
+                const int x = t + T * (m0 + k);
+                gg[k] = x < n ? __ldg(g + x) : make_float2(0.f, 0.f);
+                vv[k] = x < n ? __ldg(V + x) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int k = 0; k < CH; k++) {
+                const int m = m0 + k;
+                const int x = t + T * m;
+                if (x < n) {
+                    const float2 lam = v[m];
+                    Q[x] = cadd(qr[x], cmulc(ur[x], lam));  // += conj(lambda) u_j
+                    v[m] = cadd(gg[k], cmulc(lam, vv[k]));    // ubar_j = g + conj(V) lambda
+                } else {
+                    v[m] = make_float2(0.f, 0.f);
+                }
+            }
+        }
+#pragma unroll
+        for (int m = E / 2; m < E; m++) v[m] = make_float2(0.f, 0.f);
+        sync();  // the Q and u_j rows and the exchange line are read
+        if (t == 0 && inext < total) {
+            fence_proxy_async_smem();
+            issue_q(inext);
+        }
+        if (term > 0) {  // step 0 feeds no further column pass
+            fft_lines<M, E, -1, 1, ThreadTwiddles<M, E>, GroupSync, true, true>(va, sm, t, a.tw, &twr, sync);
+            float2 *xo = a.X + (size_t)i * M;
 #pragma unroll
             for (int m = 0; m < E; m++) xo[t + T * m] = v[m];
         }
@@ -1825,9 +1992,13 @@ static cudaError_t row_launch_th(int nrhs, const RowArgs &b, cudaStream_t s) {
         if (b.n == M && b.num_sms > 0)
             return persistent_row<row_eps_persistent_kernel<M, KIND == ROW_EPSK, TH>, RowECfg<M, TH>>(nrhs, b, s);
     }
-    if constexpr (KIND == ROW_FWD && M >= 512) {
-        if ((b.n & 1) == 0 && b.num_sms > 0)
-            return persistent_row<row_fwd_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
+    if constexpr ((KIND == ROW_FWD || KIND == ROW_ADJ) && M >= 512) {
+        if (b.num_sms > 0) {
+            if constexpr (KIND == ROW_FWD)
+                return persistent_row<row_fwd_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
+            else
+                return persistent_row<row_adj_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
+        }
     }
     dim3 grid((b.n + C::RPB - 1) / C::RPB, nrhs);
     return launch_k(row_kernel<M, KIND, TH>, grid, dim3(C::THREADS), C::SMEM, s, b.pdl != 0, b);
@@ -2085,6 +2256,7 @@ static cudaError_t row_attr() {
     set(row_kernel<M, ROW_OUT, TH>, b);
     if constexpr (M >= 512) {
         set(row_fwd_persistent_kernel<M, TH>, (int)RowPCfg<M, TH>::SMEM);
+        set(row_adj_persistent_kernel<M, TH>, (int)RowPCfg<M, TH>::SMEM);
         set(row_eps_persistent_kernel<M, false, TH>, (int)RowECfg<M, TH>::SMEM);
         set(row_eps_persistent_kernel<M, true, TH>, (int)RowECfg<M, TH>::SMEM);
     }

@@ -274,6 +274,7 @@ const char *col_variant_name(int M, bool periodic, int variant) {
     case COL_S0: return "tile S0 (lockstep, default width)";
     case COL_S1: return "tile S1 (lockstep, width/2)";
     case COL_S2: return "tile S2 (lockstep, width/4)";
+    case COL_C: return "compact, 2 columns/thread, two blocks per SM";
     case COL_P1: return "pipelined, 1 column/thread";
     case COL_P2: return "pipelined, 2 columns/thread";
     case COL_P2S: return "pipelined, 2 columns/thread, staggered";

@@ -44,7 +44,7 @@ struct RowCfg {
 // plain periodic pass keeps its code size).
 template <int M, int TC_, int L_, int MINB_ = 1, int PER_ = 0>
 struct ColShape {
-    static constexpr bool PIPE = false;  // col_kernel (ColPShape: col_pipe_kernel)
+    static constexpr bool PIPE = false, COMPACT = false;  // col_kernel (ColPShape: col_pipe_kernel)
     static constexpr int MINB = MINB_;
     static constexpr int TC = TC_;
     static constexpr int L = L_;
@@ -92,6 +92,8 @@ using ColCfgPK2 = ColShape<M, ColCfg<M>::TC, 2, 1, 2>;
 // periodic plans: lockstep with two columns per thread (M >= 32) and one
 // plus, for M >= 1024, the pipelined kernel with two columns per thread
 // (unstaggered, staggered)
+// (at M = 1024 and 2048 the two-column lockstep shape is the compact kernel)
+__host__ __device__ constexpr bool col_periodic_compact(int M) { return M == 1024 || M == 2048; }
 __host__ __device__ constexpr int col_periodic_variant_count(int M) { return M >= 1024 ? 4 : M >= 32 ? 2 : 1; }
 
 // Autotuned alternatives: variant V narrows the tile to TC >> V columns (one
@@ -126,7 +128,8 @@ __host__ __device__ constexpr int col_shape_count(int M) {
 // the pipelined kernel exists for M >= 1024
 __host__ __device__ constexpr bool col_has_pipe(int M) { return M >= 1024; }
 // For M >= 1024 there is also the pipelined kernel with one or two columns
-// per thread (P1, P2; P2S: the two columns staggered).
+// per thread (P1, P2; P2S: the two columns staggered); at M = 2048 the compact
+// kernel (C) stands in for P1.
 // At M = 4096 also the unstaggered pair with the radix split 8 x 8 x 8 x 8 (P2R8).
 __host__ __device__ constexpr int col_variant_count(int M) {
     return col_shape_count(M) + (col_has_pipe(M) ? 3 : 0) + (M >= 4096 ? 1 : 0);
@@ -134,14 +137,14 @@ __host__ __device__ constexpr int col_variant_count(int M) {
 // The variants of each M, fastest first as measured on GB300 at N = M/2
 // (variant 0 is a plan's default; tbs_autotune re-times them all):
 // S0 = col_kernel's default tile, S1/S2 = its tile narrowed once/twice.
-enum ColKind { COL_S0 = 0, COL_S1 = 1, COL_S2 = 2, COL_P1 = 3, COL_P2 = 4, COL_P2S = 5, COL_P2R8 = 6 };
+enum ColKind { COL_S0 = 0, COL_S1 = 1, COL_S2 = 2, COL_P1 = 3, COL_P2 = 4, COL_P2S = 5, COL_P2R8 = 6, COL_C = 7 };
 __host__ __device__ constexpr int col_variant_kind(int M, int v) {
     if (M >= 4096) {
         constexpr int k[5] = {COL_P2, COL_P2S, COL_P1, COL_S0, COL_P2R8};
         return k[v];
     }
     if (M == 2048) {
-        constexpr int k[5] = {COL_S1, COL_P2S, COL_P2, COL_P1, COL_S0};
+        constexpr int k[5] = {COL_C, COL_S1, COL_P2S, COL_P2, COL_S0};
         return k[v];
     }
     if (M == 1024) {
@@ -1954,6 +1957,227 @@ col_pipe_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid
 }
 
 // ---------------------------------------------------------------------------
+// compact column pass: two blocks per SM (padded grid at M = 2048, periodic
+// grid at M = 1024 and 2048)
+// ---------------------------------------------------------------------------
+// Tiles of TC = 8192 / M columns, two columns per thread (256 threads), the
+// FFT arithmetic of the other shapes.  Shared memory is one landing buffer and
+// the exchange lines, 103 KB, each used in turn:
+//   landing  input rows of the tile -> its Ghat columns (copied in once the
+//            rows are in registers, read by the spectral product) -> input
+//            rows of the next tile (during the inverse transform)
+//   lines    the two transforms' exchanges -> output rows (sent by a tensor
+//            store that the next tile's first exchange waits for)
+// so that two blocks fit an SM and one's copies, barriers and exchanges run
+// under the other's butterflies.  On the periodic grid (whole columns, no
+// Ghat) the rows land in the lines themselves, 70 KB.
+// What bounds it (N = 1024, 8 RHS): the shared-memory data pipe 65%, FMA 48%,
+// issue 58%, DRAM traffic 2.1 TB/s.  The padded pass at N = 1024 takes 219 us
+// for 16 RHS (235 with tiles of two columns, whose 16-byte rows cost twice the
+// L2 requests), 59 us for 4 x 700^2 (63); the periodic one 24.8 us at 2048^2
+// (27.8 in lockstep), 24.6 us for 4 x 1024^2 (28.8).  At M = 4096 the lines
+// leave two columns per tile and nothing is gained (71.3 against 71.7 us
+// padded, 125 against 98 us periodic); tiles of four columns with one block of
+// 512 threads: 72 and 123 us.
+template <int M, int TC_, int PER_ = 0>
+struct ColCompact : ColShape<M, TC_, 2, 2, PER_> {
+    using B_ = ColShape<M, TC_, 2, 2, PER_>;
+    static constexpr bool COMPACT = true;
+    static constexpr int G = TC_ / 2;  // column pairs: pair cg of thread t is thread t G + cg
+    // (in 16-byte units modulo 8) lanes of one quarter warp hold 8/G
+    // consecutive t of G pairs: lines 8/G apart
+    static constexpr int LSTRIDE = ((padded_len(M) + 15) / 16) * 16 + (G == 4 ? 2 : 4);
+    static constexpr int GS = B_::QSP + (G == 2 ? 2 : 0);  // Ghat column stride, likewise
+    static constexpr size_t LANDG = PER_ ? 0 : ((B_::LAND > (size_t)GS * TC_ ? B_::LAND : (size_t)GS * TC_) + 15) & ~(size_t)15;
+    static constexpr size_t SMEM = (LANDG + (size_t)LSTRIDE * TC_) * sizeof(float2) + 128;
+    static_assert(G == 1 || G == 2 || G == 4, "2, 4 or 8 columns per tile");
+    static_assert(GS % 2 == 0 && LSTRIDE % 2 == 0, "16-byte aligned columns and lines");
+    static_assert(B_::LAND <= (size_t)LSTRIDE * TC_, "the output rows fit the lines");
+};
+
+template <int M, bool CONJ, class C>
+__global__ void __launch_bounds__(C::THREADS, 2)
+col_compact_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw) {
+    constexpr int TC = C::TC, G = C::G, E = C::E, T = C::T, TILES = M / TC;
+    extern __shared__ __align__(16) float2 smem_raw[];
+    float2 *land = reinterpret_cast<float2 *>(reinterpret_cast<char *>(smem_raw) +
+                                              ((128u - (smem_u32(smem_raw) & 127u)) & 127u));
+    float2 *lines = land + C::LANDG;  // periodic grid: the rows land in the lines
+    const int n = a.n;
+    const int cg = threadIdx.x % G, t = threadIdx.x / G;
+    ThreadTwiddles<M, E> twr;
+    twr.load(a.tw, t);
+    __shared__ __align__(8) uint64_t bars[2];  // rows, Ghat
+    if (threadIdx.x == 0) {
+        mbar_init(&bars[0], 1);
+        mbar_init(&bars[1], 1);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    grid_dep_wait();  // X, the RHS flags
+    if (a.early) grid_dep_launch();  // the row pass may be scheduled beside this pass
+    const int total = TILES * a.nrhs;
+    int cached_rhs = -1;
+    bool cached_active = false;
+    auto next_active = [&](int i) {
+        while (i < total) {
+            const int r = i / TILES;
+            if (r != cached_rhs) {
+                cached_rhs = r;
+                cached_active = gate_active(a.gate, r);
+            }
+            if (cached_active) break;
+            i += gridDim.x;
+        }
+        return i;
+    };
+    constexpr unsigned GROW = C::QSP * sizeof(float2);
+    const int nx = a.xslice ? 1 : (n + C::BR - 1) / C::BR;
+    const unsigned xbytes = (unsigned)((a.xslice ? n : nx * C::BR) * TC * sizeof(float2));
+    // thread 0 issues every copy; each first checks the copy rules (a
+    // violation sets the error word and arms a barrier that never completes)
+    auto load_rows = [&](int i) {
+        const int x0 = (i % TILES) * TC, r = i / TILES;
+        if ((smem_u32(land) & 127u) != 0 || ((x0 * (int)sizeof(float2)) & 15) != 0) {
+            if (a.err) atomicExch(a.err, 2);
+            mbar_arrive_expect_tx(&bars[0], 16u);
+            return;
+        }
+        mbar_arrive_expect_tx(&bars[0], xbytes + a.extra_tx);
+        for (int q = 0; q < nx; q++) {
+            if (a.xslice)
+                tma_load_3d(land, &tmx, x0, 0, r * (n / a.xslice), &bars[0]);
+            else
+                tma_load_3d(land + (size_t)q * C::BR * TC, &tmx, x0, q * C::BR, r, &bars[0]);
+        }
+    };
+    auto load_ghat = [&](int i) {
+        const int x0 = (i % TILES) * TC;
+        if ((GROW & 15u) != 0 || (reinterpret_cast<uintptr_t>(a.ghq) & 15u) != 0) {
+            if (a.err) atomicExch(a.err, 2);
+            mbar_arrive_expect_tx(&bars[1], 16u);
+            return;
+        }
+        mbar_arrive_expect_tx(&bars[1], TC * GROW);
+        for (int c = 0; c < TC; c++) {
+            const int kx = x0 + c;
+            const int kxq = kx <= M / 2 ? kx : M - kx;  // column kx of Ghat = quadrant row kxq
+            bulk_load(land + c * C::GS, a.ghq + (size_t)kxq * C::QSP, GROW, &bars[1]);
+        }
+    };
+    auto store_rows = [&](int i) {
+        const int x0 = (i % TILES) * TC, r = i / TILES;
+        for (int q = 0; q < nx; q++) {
+            if (a.xslice)
+                tma_store_3d(&tmw, x0, 0, r * (n / a.xslice), lines);
+            else
+                tma_store_3d(&tmw, x0, q * C::BR, r, lines + (size_t)q * C::BR * TC);
+        }
+        bulk_commit();
+    };
+    const Lines<2, true> sm{lines + 2 * cg * C::LSTRIDE, C::LSTRIDE};
+    int cur = next_active(blockIdx.x);
+    if (threadIdx.x == 0 && cur < total) load_rows(cur);
+    col_stop(a.stop, a.nrhs);
+    unsigned ph = 0u;  // both barriers complete once per tile
+    while (cur < total) {
+        const int nxt = next_active(cur + gridDim.x);
+        const bool ok = mbar_wait_bounded(&bars[0], ph, a.wait_ns, a.err);
+        float2 v[2][E];
+        col_load<C, M>(v, land, TC, n, t, 2 * cg);
+        if (threadIdx.x == 0) bulk_wait_read_all();  // the previous tile's store has read the lines
+        // the rows are in registers, the lines free
+        if (__syncthreads_or(!ok)) {
+            // a copy never completed: give its bytes one more bounded chance
+            // to land, let the stores finish, then leave (error word set)
+            if (threadIdx.x == 0) {
+                mbar_wait_bounded(&bars[0], ph, a.wait_ns, nullptr);
+                bulk_wait_all();
+            }
+            return;
+        }
+        if (!C::PER && threadIdx.x == 0) {
+            fence_proxy_async_smem();
+            load_ghat(cur);
+        }
+        fft_lines<M, E, -1, 2, ThreadTwiddles<M, E>, BlockSync, true, !C::PER, true>(v, sm, t, a.tw, &twr);
+        if constexpr (C::PER) {
+            const int x0 = (cur % TILES) * TC;
+            auto multiply = [&](auto ks) {
+                constexpr bool KS = decltype(ks)::value;
+#pragma unroll
+                for (int l = 0; l < 2; l++) {
+                    const int kx = x0 + 2 * cg + l;
+                    const float ix = (float)(kx < M / 2 ? kx : kx - M);
+#pragma unroll
+                    for (int m = 0; m < E; m++) {
+                        const int ky = t + T * m;
+                        v[l][m] = cmul(v[l][m], periodic_spectrum<KS>(a, ix, (float)(ky < M / 2 ? ky : ky - M)));
+                    }
+                }
+            };
+            // with the k-space potential from the RHS's second term on (its
+            // first applies G only)
+            if constexpr (C::KS) {
+                if (a.stop.st || (a.gate.st && a.gate.st[cur / TILES].terms > 0))
+                    multiply(std::true_type{});
+                else
+                    multiply(std::false_type{});
+            } else {
+                multiply(std::false_type{});
+            }
+            __syncthreads();  // the forward transform's exchanges are read
+        } else {
+            const bool okg = mbar_wait_bounded(&bars[1], ph, a.wait_ns, a.err);
+#pragma unroll
+            for (int l = 0; l < 2; l++) {
+                const float2 *gcol = land + (2 * cg + l) * C::GS;
+#pragma unroll
+                for (int m = 0; m < E; m++) {
+                    const int ky = t + T * m;
+                    const float2 g = gcol[ky <= M / 2 ? ky : M - ky];
+                    v[l][m] = CONJ ? cmulc(v[l][m], g) : cmul(v[l][m], g);
+                }
+            }
+            // Ghat is read, and the forward transform's exchanges
+            if (__syncthreads_or(!okg)) {
+                if (threadIdx.x == 0) {
+                    mbar_wait_bounded(&bars[1], ph, a.wait_ns, nullptr);
+                    bulk_wait_all();
+                }
+                return;
+            }
+        }
+        ph ^= 1u;
+        if (!C::PER && threadIdx.x == 0 && nxt < total) {
+            fence_proxy_async_smem();
+            load_rows(nxt);
+        }
+        fft_lines<M, E, +1, 2, ThreadTwiddles<M, E>, BlockSync, true, false, true>(v, sm, t, a.tw, &twr);
+        __syncthreads();  // the inverse transform's exchanges are read
+#pragma unroll
+        for (int m = 0; m < (C::PER ? E : E / 2); m++) {
+            const int y = t + T * m;
+            if (y < n)
+                *reinterpret_cast<float4 *>(lines + (size_t)y * TC + 2 * cg) =
+                    make_float4(v[0][m].x, v[0][m].y, v[1][m].x, v[1][m].y);
+        }
+        fence_proxy_async_smem();  // this thread's output rows, for the tensor store
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            store_rows(cur);
+            if (C::PER && nxt < total) {
+                bulk_wait_read_all();
+                fence_proxy_async_smem();
+                load_rows(nxt);
+            }
+        }
+        cur = nxt;
+    }
+    if (threadIdx.x == 0) bulk_wait_all();
+}
+
+// ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
 // Resident blocks per SM of a persistent row kernel (per process: the
@@ -2047,7 +2271,10 @@ static cudaError_t col_launch(int nrhs, const ColArgs &a, const ColMaps *maps, c
     // one block per tile, and per stop test, up to the resident ones
     const int tiles = (M / C::TC) * nrhs, work = tiles + (a.stop.st ? nrhs : 0);
     const int grid = work < a.num_sms ? work : a.num_sms;
-    if constexpr (C::PIPE) {
+    if constexpr (C::COMPACT) {
+        return launch_k(col_compact_kernel<M, CONJ, C>, dim3(grid), dim3(C::THREADS), C::SMEM, s, a.pdl != 0, b,
+                        maps->x, maps->w);
+    } else if constexpr (C::PIPE) {
         return launch_k(col_pipe_kernel<M, CONJ, C::L, C::STAG, C::PERK, C::RS>, dim3(grid), dim3(C::THREADS), C::SMEM,
                         s, a.pdl != 0, b, maps->x, maps->w);
     } else {
@@ -2064,7 +2291,11 @@ static cudaError_t with_col_variant(int variant, int nrhs, F f) {
         if (col_narrow(M, nrhs, false)) return f(ColNarrow<M>{});
     const int kind = col_variant_kind(M, variant);
     if constexpr (col_has_pipe(M)) {
-        if (kind == COL_P1) return f(ColPShape<M, 1>{});
+        if constexpr (M == 2048) {
+            if (kind == COL_C) return f(ColCompact<M, 8192 / M>{});
+        } else {
+            if (kind == COL_P1) return f(ColPShape<M, 1>{});
+        }
         if (kind == COL_P2) return f(ColPShape<M, 2>{});
         if (kind == COL_P2S) return f(ColPShape<M, 2, true>{});
         if constexpr (M >= 4096)
@@ -2130,8 +2361,11 @@ template <int M, class F>
 static cudaError_t with_col_variant_per(int variant, int nrhs, bool ks, F f) {
     if constexpr (col_narrow(M, 1, true))
         if (variant == 0 && col_narrow(M, nrhs, true)) return ks ? f(ColNarrowP<M, 2>{}) : f(ColNarrowP<M, 1>{});
-    // fastest first as measured on GB300 at M = 4096: two columns per thread,
-    // then one (the only shape below M = 32)
+    // fastest first as measured on GB300: at M = 1024 and 2048 the compact
+    // kernel, else two columns per thread of col_kernel, then one (the only
+    // shape below M = 32)
+    if constexpr (col_periodic_compact(M))
+        if (variant == 0) return ks ? f(ColCompact<M, 8192 / M, 2>{}) : f(ColCompact<M, 8192 / M, 1>{});
     if constexpr (col_periodic_variant_count(M) > 1) {
         if (variant == 0) return ks ? f(ColCfgPK2<M>{}) : f(ColCfgP2<M>{});
         if (variant == 1) return ks ? f(ColCfgPK<M>{}) : f(ColCfgP<M>{});
@@ -2176,7 +2410,9 @@ template <int M, class C = ColCfg<M>>
 static int col_blocks_per_sm() {
     int nb = 0;
     cudaError_t e;
-    if constexpr (C::PIPE)
+    if constexpr (C::COMPACT)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, col_compact_kernel<M, false, C>, C::THREADS, C::SMEM);
+    else if constexpr (C::PIPE)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, col_pipe_kernel<M, false, C::L, C::STAG, C::PERK, C::RS>,
                                                           C::THREADS, C::SMEM);
     else
@@ -2204,7 +2440,15 @@ int col_resident_blocks_m(int variant, int nrhs, bool periodic) {
 
 template <int M, class C = ColCfg<M>>
 static cudaError_t col_attr() {
-    if constexpr (C::PIPE) {
+    if constexpr (C::COMPACT) {
+        cudaError_t e = cudaFuncSetAttribute(col_compact_kernel<M, false, C>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+        if constexpr (!C::PER)  // the periodic grid has no adjoint pass
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(col_compact_kernel<M, true, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)C::SMEM);
+        return e;
+    } else if constexpr (C::PIPE) {
         cudaError_t e = cudaFuncSetAttribute(col_pipe_kernel<M, false, C::L, C::STAG, C::PERK, C::RS>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess || C::PERK) return e;  // the periodic grid has no adjoint pass
@@ -2225,7 +2469,7 @@ cudaError_t set_col_smem_attr_m() {
     cudaError_t e = cudaSuccess;
     auto per = [](auto c) {
         using CC = decltype(c);
-        if constexpr (CC::PIPE)
+        if constexpr (CC::PIPE || CC::COMPACT)
             return col_attr<M, CC>();
         else
             return cudaFuncSetAttribute(col_kernel<M, false, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -311,10 +311,11 @@ void drop_graphs(tbs_plan_s *p) {
 bool early_columns(const tbs_plan_s *p) { return (size_t)p->nrhs * p->n * p->M <= (size_t)512 * 1024; }
 
 tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
-    TBS_CK(cudaMemsetAsync(p->state, 0, sizeof(RhsState) * p->nrhs, s));
-    TBS_CK(cudaMemsetAsync(p->err, 0, 4 * sizeof(int), s));
     RowArgs ra = row_args(p);
     ColArgs ca = col_args(p);
+    ra.clear = p->state;
+    ra.clear_words = (int)(sizeof(RhsState) / sizeof(int)) * p->nrhs;
+    ra.clear_err = p->err;
     TBS_CK(timed_row(p, ROW_SRC, ra, s));
     StopArgs sa;
     sa.part = p->part;
@@ -399,7 +400,25 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
             if (t == p->d.max_terms - 1 || !fused) TBS_CK(launch_stop(p->nrhs, sa, s));
         }
     }
-    TBS_CK(launch_info(p->nrhs, p->state, p->err, p->info_dev, s));
+    return TBS_OK;
+}
+
+bool is_device_ptr(const void *ptr);
+
+// The outputs of the solve enqueued on s: psi and the records to the caller's
+// buffers.  Small fields travel in the kernel that writes the records (a
+// 256^2 solve is three launches shorter); larger ones by a device copy.
+tbs_status enqueue_outputs(tbs_plan_s *p, float *psi, tbs_solve_info *info, bool device_info, cudaStream_t s) {
+    const size_t count = (size_t)p->nrhs * p->n * p->n;
+    const bool direct = device_info && (reinterpret_cast<uintptr_t>(info) & 7) == 0;
+    const bool fused = is_device_ptr(psi) && count % 2 == 0 && (reinterpret_cast<uintptr_t>(psi) & 15) == 0 && count <= ((size_t)1 << 19);
+    if (!fused)
+        TBS_CK(cudaMemcpyAsync(psi, p->psi, sizeof(float2) * count, cudaMemcpyDeviceToDevice, s));
+    TBS_CK(launch_finish(p->nrhs, p->state, p->err, direct ? (void *)info : p->info_dev, p->psi,
+                         fused ? (float2 *)psi : nullptr, count, s));
+    if (!direct)
+        TBS_CK(cudaMemcpyAsync(info, p->info_dev, sizeof(tbs_solve_info) * p->nrhs,
+                               device_info ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
     return TBS_OK;
 }
 
@@ -814,8 +833,16 @@ tbs_status tbs_set_medium(tbs_plan_t p, const float *c, const float *alpha, doub
     if (!p || !c) return fail(TBS_ERR_INVALID_ARG, "plan and c must not be NULL");
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nn = (size_t)p->n * p->n;
-    TBS_CK(cudaMemcpyAsync(p->c, c, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    if (alpha) TBS_CK(cudaMemcpyAsync(p->alpha, alpha, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
+    // the kernel that forms V also keeps copies of c and alpha (for gradients);
+    // what it cannot read is copied first
+    if (!is_device_ptr(c)) {
+        TBS_CK(cudaMemcpyAsync(p->c, c, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
+        c = p->c;
+    }
+    if (alpha && !is_device_ptr(alpha)) {
+        TBS_CK(cudaMemcpyAsync(p->alpha, alpha, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
+        alpha = p->alpha;
+    }
     p->have_alpha = alpha != nullptr;
     p->ypow = y_pow;
     p->fref = f_ref_hz;
@@ -826,12 +853,12 @@ tbs_status tbs_set_medium(tbs_plan_t p, const float *c, const float *alpha, doub
     }
     p->tdel = tdel;
     if (p->cbs_auto) {
-        TBS_CK(launch_medium((int)nn, p->c, alpha ? p->alpha : nullptr, p->omega, p->d.c0, tdel, 0.0, p->V, s));
+        TBS_CK(launch_medium((int)nn, c, alpha, p->omega, p->d.c0, tdel, 0.0, p->V, p->c, p->alpha, s));
         tbs_status st = cbs_auto_eps(p, s);
         if (st != TBS_OK) return st;
         TBS_CK(launch_shift_potential((int)nn, p->eps, p->V, s));  // U - i eps
     } else {
-        TBS_CK(launch_medium((int)nn, p->c, alpha ? p->alpha : nullptr, p->omega, p->d.c0, tdel, p->eps, p->V, s));
+        TBS_CK(launch_medium((int)nn, c, alpha, p->omega, p->d.c0, tdel, p->eps, p->V, p->c, p->alpha, s));
     }
     p->have_medium = true;
     p->medium_from_c = true;
@@ -972,10 +999,8 @@ tbs_status tbs_solve(tbs_plan_t p, float *psi, tbs_solve_info *info, void *strea
         tbs_status st = enqueue_solve(p, s, false);
         if (st != TBS_OK) return st;
     }
-    const size_t nn = (size_t)p->n * p->n;
-    TBS_CK(cudaMemcpyAsync(psi, p->psi, sizeof(float2) * p->nrhs * nn, cudaMemcpyDeviceToDevice, s));
-    TBS_CK(cudaMemcpyAsync(info, p->info_dev, sizeof(tbs_solve_info) * p->nrhs,
-                           is_device_ptr(info) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+    tbs_status st = enqueue_outputs(p, psi, info, is_device_ptr(info), s);
+    if (st != TBS_OK) return st;
     p->solved = true;
     return TBS_OK;
 }
@@ -1029,15 +1054,9 @@ tbs_status tbs_batch_create(const tbs_plan_t *plans, int32_t n_plans, float *con
     if (e == cudaSuccess) e = cudaEventRecord(b->events[0], b->origin);
     for (int i = 0; e == cudaSuccess && st == TBS_OK && i < n_plans; i++) {
         tbs_plan_s *p = b->plans[i];
-        const size_t nn = (size_t)p->n * p->n;
         if ((e = cudaStreamWaitEvent(p->cap, b->events[0], 0)) != cudaSuccess) break;
         if ((st = enqueue_solve(p, p->cap, true)) != TBS_OK) break;
-        if ((e = cudaMemcpyAsync(psi[i], p->psi, sizeof(float2) * p->nrhs * nn, cudaMemcpyDeviceToDevice,
-                                 p->cap)) != cudaSuccess)
-            break;
-        if ((e = cudaMemcpyAsync(info[i], p->info_dev, sizeof(tbs_solve_info) * p->nrhs,
-                                 cudaMemcpyDeviceToDevice, p->cap)) != cudaSuccess)
-            break;
+        if ((st = enqueue_outputs(p, psi[i], info[i], true, p->cap)) != TBS_OK) break;
         if ((e = cudaEventRecord(b->events[i + 1], p->cap)) != cudaSuccess) break;
         e = cudaStreamWaitEvent(b->origin, b->events[i + 1], 0);
     }
@@ -1112,12 +1131,15 @@ tbs_status tbs_apply_green(tbs_plan_t p, const float *f, float *out, int32_t con
     if (!p || !f || !out) return fail(TBS_ERR_INVALID_ARG, "NULL argument to tbs_apply_green");
     if (f == out) return fail(TBS_ERR_INVALID_ARG, "f and out may not alias");
     cudaStream_t s = (cudaStream_t)stream;
-    TBS_CK(cudaMemsetAsync(p->err, 0, sizeof(int), s));  // read back by tbs_device_error
     RowArgs ra = row_args(p);
     ra.src = (const float2 *)f;
     ra.psi = (float2 *)out;
+    ra.clear_err = p->err;  // read back by tbs_device_error
     ColArgs ca = col_args(p);
     TBS_CK(timed_row(p, ROW_SRC, ra, s));
+    // each pass a programmatic dependent of the one before, as in a solve
+    ca.pdl = early_columns(p);
+    ra.pdl = 1;
     TBS_CK(timed_col(p, conj_kernel != 0, ca, s));
     TBS_CK(timed_row(p, ROW_OUT, ra, s));
     return TBS_OK;

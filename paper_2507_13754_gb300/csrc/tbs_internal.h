@@ -105,6 +105,11 @@ struct RowArgs {
     unsigned long long wait_ns;  // limit of those waits
     int num_sms;        // SM count (persistent steady-state pass), or 0: one block per row
     int nrhs;           // set by the launcher
+    // ROW_SRC: words it sets to zero before anything else of the call reads
+    // them (the RHS states; the error words), or none
+    void *clear;
+    int clear_words;
+    int *clear_err;     // 4 words, or null
 };
 
 struct ColArgs {
@@ -166,10 +171,15 @@ cudaError_t launch_stop(int nrhs, const StopArgs &a, cudaStream_t s);
 // else *j -= steps; then the WHILE condition is set to (*j >= 0).
 cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphConditionalHandle h, bool init, int steps,
                             cudaStream_t s);
-cudaError_t launch_info(int nrhs, const RhsState *st, const int *err, void *info_dev, cudaStream_t s);
-// V = p^2 - k0^2 - i eps_shift (eps_shift = 0 except on the periodic grid)
-cudaError_t launch_medium(int count, const float *c, const float *alpha, double omega,
-                          double c0, double tdel, double eps_shift, float2 *V, cudaStream_t s);
+// A solve's outputs: its records to info (8-byte aligned device memory) and, in
+// the same kernel, psi copied to out (out null: records only; out 16-byte
+// aligned, count even).
+cudaError_t launch_finish(int nrhs, const RhsState *st, const int *err, void *info, const float2 *psi, float2 *out,
+                          size_t count, cudaStream_t s);
+// V = p^2 - k0^2 - i eps_shift (eps_shift = 0 except on the periodic grid);
+// c and alpha (or null) are also copied to c_copy and alpha_copy
+cudaError_t launch_medium(int count, const float *c, const float *alpha, double omega, double c0, double tdel,
+                          double eps_shift, float2 *V, float *c_copy, float *alpha_copy, cudaStream_t s);
 // *out = the bits of max |V + i eps_shift| over `count` points (FP64)
 cudaError_t launch_potential_max(int count, const float2 *V, double eps_shift, unsigned long long *out,
                                  cudaStream_t s);

@@ -65,15 +65,21 @@ __global__ void adj_loop_kernel(int nrhs, const RhsState *st, int *jdev, cudaGra
     cudaGraphSetConditional(h, j >= 0 ? 1u : 0u);
 }
 
-__global__ void info_kernel(int nrhs, const RhsState *st, const int *err, InfoOut *out) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= nrhs) return;
-    out[r].terms = st[r].terms;
-    // error word: 1 -> TBS_WAIT_TIMEOUT (4), 2 -> TBS_COPY_CHECK_FAILED (5)
-    out[r].status = (err && *err) ? 3 + *err : st[r].status;
-    out[r].residual = st[r].residual;
-    out[r].term_norm_max = st[r].tmax;
-    out[r].psi_norm = st[r].psi_norm;
+// The records (one thread per RHS of the first blocks) and the copy of psi,
+// float4 by float4: one launch where a kernel and two copies took three.
+__global__ void __launch_bounds__(256) finish_kernel(int nrhs, const RhsState *st, const int *err, InfoOut *out,
+                                                     const float4 *__restrict__ psi, float4 *__restrict__ dst,
+                                                     int count4) {
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i < nrhs) {
+        out[i].terms = st[i].terms;
+        // error word: 1 -> TBS_WAIT_TIMEOUT (4), 2 -> TBS_COPY_CHECK_FAILED (5)
+        out[i].status = (err && *err) ? 3 + *err : st[i].status;
+        out[i].residual = st[i].residual;
+        out[i].term_norm_max = st[i].tmax;
+        out[i].psi_norm = st[i].psi_norm;
+    }
+    for (int j = i; j < count4; j += gridDim.x * 256) dst[j] = psi[j];
 }
 
 // ---------------------------------------------------------------------------
@@ -87,13 +93,15 @@ __global__ void info_kernel(int nrhs, const RhsState *st, const int *err, InfoOu
 // for c within a factor two of c0), Re V = d (2 k0 + d) - alpha^2 and
 // Im V = 2 Re p alpha - eps_shift, so FP32 keeps V to a few ulp of itself
 // (an FP64 evaluation was FP64-issue-bound on this GPU: ~0.1 ms at 2048^2).
-__global__ void medium_kernel(int count, const float *__restrict__ c, const float *__restrict__ alpha,
+__global__ void medium_kernel(int count, const float *c, const float *alpha,
                               float omega, float k0, float c0, float tdel, float eps_shift,
-                              float2 *__restrict__ V) {
+                              float2 *__restrict__ V, float *c_copy, float *alpha_copy) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const float ci = c[i];
     const float al = alpha ? alpha[i] : 0.f;
+    c_copy[i] = ci;
+    if (alpha) alpha_copy[i] = al;
     const float d = fmaf(al, tdel, omega * (c0 - ci) / (ci * c0));
     const float pr = k0 + d;
     V[i] = make_float2(fmaf(d, fmaf(2.f, k0, d), -al * al), fmaf(2.f * pr, al, -eps_shift));
@@ -341,15 +349,20 @@ cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphCondi
     return cudaGetLastError();
 }
 
-cudaError_t launch_info(int nrhs, const RhsState *st, const int *err, void *info_dev, cudaStream_t s) {
-    info_kernel<<<(nrhs + 127) / 128, 128, 0, s>>>(nrhs, st, err, (InfoOut *)info_dev);
+cudaError_t launch_finish(int nrhs, const RhsState *st, const int *err, void *info, const float2 *psi, float2 *out,
+                          size_t count, cudaStream_t s) {
+    const int count4 = out ? (int)(count / 2) : 0;
+    const int work = count4 > nrhs ? count4 : nrhs;
+    finish_kernel<<<(work + 255) / 256, 256, 0, s>>>(nrhs, st, err, (InfoOut *)info, (const float4 *)psi,
+                                                     (float4 *)out, count4);
     return cudaGetLastError();
 }
 
 cudaError_t launch_medium(int count, const float *c, const float *alpha, double omega, double c0,
-                          double tdel, double eps_shift, float2 *V, cudaStream_t s) {
+                          double tdel, double eps_shift, float2 *V, float *c_copy, float *alpha_copy,
+                          cudaStream_t s) {
     medium_kernel<<<(count + 255) / 256, 256, 0, s>>>(count, c, alpha, (float)omega, (float)(omega / c0), (float)c0,
-                                                      (float)tdel, (float)eps_shift, V);
+                                                      (float)tdel, (float)eps_shift, V, c_copy, alpha_copy);
     return cudaGetLastError();
 }
 

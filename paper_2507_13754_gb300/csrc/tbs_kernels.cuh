@@ -452,6 +452,12 @@ row_kernel(RowArgs a) {
     }
     grid_dep_launch();  // the next kernel may be scheduled once every row block runs
     if constexpr (KIND == ROW_FWD || KIND == ROW_EPS || KIND == ROW_EPSK) mark_before_row(a);
+    if constexpr (KIND == ROW_SRC) {  // a solve or G application begins: zero its state and error words
+        if (blockIdx.x == 0 && blockIdx.y == 0) {
+            for (int i = threadIdx.x; i < a.clear_words; i += C::THREADS) reinterpret_cast<int *>(a.clear)[i] = 0;
+            if (a.clear_err && threadIdx.x < 4) a.clear_err[threadIdx.x] = 0;
+        }
+    }
     TBS_ROW_PHASE_DECL
     if (!gate_active(a.gate, rhs)) {
         if (bulk) {

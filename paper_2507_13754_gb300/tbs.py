@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "_lib", "libtbs.so")
@@ -227,7 +228,13 @@ def tbs_apply_green_noalloc(n, ghat_ptr, f_ptr, out_ptr, conj_kernel=0, stream=0
 
 def tbs_synthesize(entries, n_rhs, x0, y0, sx, sy, nx, ny, t0, dt, n_t, out_ptr, stream=0):
     """entries: [(field_ptr, n, dx, freq_hz, weight)]; out [n_rhs][ny][nx][n_t] complex64."""
-    arr = (tbs_synth_freq * len(entries))(*[tbs_synth_freq(*e) for e in entries])
+    # one pack of all records (a ctypes structure per entry costs a microsecond)
+    arr = (tbs_synth_freq * len(entries))()
+    try:
+        struct.pack_into("@" + "Pi0dddd" * len(entries), arr, 0, *[v for e in entries for v in e])
+    except struct.error:  # numbers in other forms
+        for a, (ptr, n, dx, f, w) in zip(arr, entries):
+            a.field, a.n, a.dx, a.freq_hz, a.weight = ptr, n, float(dx), float(f), float(w)
     _check("tbs_synthesize", load_library().tbs_synthesize(arr, len(entries), n_rhs, x0, y0, sx, sy, nx, ny,
                                                             t0, dt, n_t, out_ptr, stream))
 
@@ -241,11 +248,10 @@ def synthesize(fields, dxs, freqs_hz, weights, origin, step, counts, t0, dt, n_t
     if not (len(fields) == len(dxs) == len(freqs_hz) == len(weights)) or not fields:
         raise ValueError("one dx, frequency and weight per field")
     n_rhs = fields[0].shape[0]
-    entries = []
+    entries, c64 = [], torch.complex64
     for k, f in enumerate(fields):
         n = f.shape[-1]
-        entries.append((_dev_ptr(f, torch.complex64, (n_rhs, n, n), "fields[%d]" % k), n, float(dxs[k]),
-                        float(freqs_hz[k]), float(weights[k])))
+        entries.append((_dev_ptr(f, c64, (n_rhs, n, n), ("fields[%d]", k)), n, dxs[k], freqs_hz[k], weights[k]))
     nx, ny = counts
     if out is None:
         out = torch.empty((n_rhs, ny, nx, n_t), dtype=torch.complex64, device="cuda")
@@ -399,24 +405,35 @@ def tbs_destroy(plan):
 
 # ---- torch marshalling -------------------------------------------------------
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream(stream=None):
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    # the current stream's handle without building a Stream object
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _dev_ptr(t, dtype, shape, name):
+    """Address of a contiguous CUDA tensor of this dtype and shape (a tuple).
+    name: what an error calls it, text or (format, value)."""
     torch = _torch()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
-        raise TypeError("%s must be a CUDA tensor" % name)
-    if t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
+        raise TypeError("%s must be a CUDA tensor" % (name if isinstance(name, str) else name[0] % name[1]))
+    if t.dtype != dtype or t.shape != shape or not t.is_contiguous():
         raise ValueError("%s must be a contiguous %s tensor of shape %s (got %s %s)"
-                         % (name, dtype, tuple(shape), t.dtype, tuple(t.shape)))
+                         % (name if isinstance(name, str) else name[0] % name[1], dtype, tuple(shape), t.dtype,
+                            tuple(t.shape)))
     return t.data_ptr()
 
 

@@ -753,7 +753,6 @@ static tbs_status plan_create(const tbs_plan_desc *d, void *workspace, size_t wo
             abl_host[i] = (float)(1.0 / (1.0 + exp(-d->abl_zeta * (edge * d->dx - 0.5 * mu))));
         }
     }
-    p->col_variant = col_default_variant(p->M, p->periodic);
     int dev = 0;
     if ((e = cudaGetDevice(&dev)) == cudaSuccess)
         e = cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, dev);

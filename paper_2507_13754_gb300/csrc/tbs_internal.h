@@ -221,7 +221,5 @@ void set_last_error(const char *msg);
 // resident column-pass blocks per SM (after set_col_smem_attr), for the
 // persistent grid (tbs_kernels.cu)
 int col_resident_blocks_per_sm(int M, int variant, int nrhs, bool periodic = false);
-// the variant a plan starts with
-int col_default_variant(int M, bool periodic);
 
 }  // namespace tbs

@@ -309,12 +309,6 @@ cudaError_t launch_col(int M, int nrhs, bool cj, const ColArgs &a, const ColMaps
     return cudaErrorInvalidValue;
 }
 
-int col_default_variant(int M, bool periodic) {
-    // M = 512: tiles of 2 columns instead of 8, four times the blocks (the
-    // pass at N = 256 with 1 / 4 / 8 RHS 10.3 / 16.4 / 26.8 -> 6.3 / 10.3 / 14.5 us)
-    return !periodic && M == 512 ? 2 : 0;
-}
-
 int col_resident_blocks_per_sm(int M, int variant, int nrhs, bool periodic) {
 #define TBS_CASE(MM) \
     case MM: return col_resident_blocks_m<MM>(variant, nrhs, periodic);

@@ -151,7 +151,12 @@ __host__ __device__ constexpr int col_variant_kind(int M, int v) {
         constexpr int k[6] = {COL_S2, COL_S1, COL_P2S, COL_P2, COL_P1, COL_S0};
         return k[v];
     }
-    return v;  // S0, S1, S2 in order
+    if (M == 512) {  // tiles of 2 columns, four times the blocks of 8: the pass at
+                     // N = 256 with 1 / 4 / 8 RHS 10.3 / 16.4 / 26.8 -> 6.3 / 10.3 / 14.5 us
+        constexpr int k[3] = {COL_S2, COL_S1, COL_S0};
+        return k[v];
+    }
+    return v;  // one shape, S0
 }
 static_assert(col_variant_count(1024) <= MAX_COL_VARIANTS && col_variant_count(512) <= MAX_COL_VARIANTS &&
                   col_periodic_variant_count(4096) <= MAX_COL_VARIANTS,

@@ -138,7 +138,7 @@ NoallocDevice *noalloc_device(cudaStream_t s, cudaError_t *err) {
             *err = e;
             return nullptr;
         }
-        d.grid[i] = sms * col_resident_blocks_per_sm(M, col_default_variant(M, false), 1);
+        d.grid[i] = sms * col_resident_blocks_per_sm(M, 0, 1);
     }
     d.ready = true;
     return &d;
@@ -195,12 +195,11 @@ extern "C" tbs_status tbs_apply_green_noalloc(int32_t n, const float *ghat, cons
         return na_fail(TBS_ERR_CUDA, "tbs_apply_green_noalloc: error word", e);
     ra.err = errw;
     ca.err = errw;
-    const int variant = col_default_variant(M, false);
     ColMaps maps;  // host-side descriptors, passed by value to the kernel
-    if ((e = col_tensor_maps(&maps, X, W, n, M, 1, variant)) != cudaSuccess)
+    if ((e = col_tensor_maps(&maps, X, W, n, M, 1, 0)) != cudaSuccess)
         return na_fail(TBS_ERR_CUDA, "tbs_apply_green_noalloc: tensor maps", e);
     if ((e = launch_row(ROW_SRC, M, 1, ra, s)) != cudaSuccess ||
-        (e = launch_col(M, 1, conj_kernel != 0, ca, &maps, variant, s)) != cudaSuccess ||
+        (e = launch_col(M, 1, conj_kernel != 0, ca, &maps, 0, s)) != cudaSuccess ||
         (e = launch_row(ROW_OUT, M, 1, ra, s)) != cudaSuccess)
         return na_fail(TBS_ERR_CUDA, "tbs_apply_green_noalloc: launch failed", e);
     return TBS_OK;

@@ -497,6 +497,7 @@ tbs_status enqueue_adjoint_ckpt(tbs_plan_s *p, cudaStream_t s, int tmax) {
     RowArgs rv = row_args(p), ro = row_args(p);
     ro.U = rv.U = nullptr;
     rv.X = p->Xs;
+    ra.pdl = ro.pdl = 1;  // each follows its column pass programmatically, as in the stored sweep
     ColArgs cr = col_args(p);
     const int K = p->ck, jtop = tmax - 2;
     for (int c = jtop >= 0 ? jtop / K : -1; c >= 0; c--) {

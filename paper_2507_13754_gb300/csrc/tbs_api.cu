@@ -834,12 +834,14 @@ tbs_status tbs_set_medium(tbs_plan_t p, const float *c, const float *alpha, doub
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nn = (size_t)p->n * p->n;
     // the kernel that forms V also keeps copies of c and alpha (for gradients);
-    // what it cannot read is copied first
-    if (!is_device_ptr(c)) {
+    // what it cannot read (host memory, addresses off a float's boundary) is
+    // copied first
+    auto readable = [](const float *f) { return is_device_ptr(f) && (reinterpret_cast<uintptr_t>(f) & 3) == 0; };
+    if (!readable(c)) {
         TBS_CK(cudaMemcpyAsync(p->c, c, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
         c = p->c;
     }
-    if (alpha && !is_device_ptr(alpha)) {
+    if (alpha && !readable(alpha)) {
         TBS_CK(cudaMemcpyAsync(p->alpha, alpha, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
         alpha = p->alpha;
     }

@@ -72,6 +72,7 @@ void tbs::set_last_error(const char *msg) { snprintf(g_err, sizeof(g_err), "%s",
 struct tbs_plan_s {
     tbs_plan_desc d;
     int n = 0, M = 0, nrhs = 0, num_sms = 1;  // num_sms: SM count of the device
+    int device = 0;                  // the device current when the plan was made
     double omega = 0, k0 = 0;
     // device buffers
     void *base = nullptr;            // every fixed-size buffer below is carved from it
@@ -403,15 +404,23 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     return TBS_OK;
 }
 
-bool is_device_ptr(const void *ptr);
+// Whether the plan's kernels may use ptr as an array of `align`-byte elements.
+bool kernel_may_use(const tbs_plan_s *p, const void *ptr, size_t align) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return kernel_reaches(at.type, at.device, p->device) && reinterpret_cast<uintptr_t>(ptr) % align == 0;
+}
 
 // The outputs of the solve enqueued on s: psi and the records to the caller's
 // buffers.  Small fields travel in the kernel that writes the records (a
 // 256^2 solve is three launches shorter); larger ones by a device copy.
 tbs_status enqueue_outputs(tbs_plan_s *p, float *psi, tbs_solve_info *info, bool device_info, cudaStream_t s) {
     const size_t count = (size_t)p->nrhs * p->n * p->n;
-    const bool direct = device_info && (reinterpret_cast<uintptr_t>(info) & 7) == 0;
-    const bool fused = is_device_ptr(psi) && count % 2 == 0 && (reinterpret_cast<uintptr_t>(psi) & 15) == 0 && count <= ((size_t)1 << 19);
+    const bool direct = device_info && kernel_may_use(p, info, 8);
+    const bool fused = count % 2 == 0 && count <= ((size_t)1 << 19) && kernel_may_use(p, psi, 16);
     if (!fused)
         TBS_CK(cudaMemcpyAsync(psi, p->psi, sizeof(float2) * count, cudaMemcpyDeviceToDevice, s));
     TBS_CK(launch_finish(p->nrhs, p->state, p->err, direct ? (void *)info : p->info_dev, p->psi,
@@ -754,9 +763,8 @@ static tbs_status plan_create(const tbs_plan_desc *d, void *workspace, size_t wo
             abl_host[i] = (float)(1.0 / (1.0 + exp(-d->abl_zeta * (edge * d->dx - 0.5 * mu))));
         }
     }
-    int dev = 0;
-    if ((e = cudaGetDevice(&dev)) == cudaSuccess)
-        e = cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, dev);
+    if ((e = cudaGetDevice(&p->device)) == cudaSuccess)
+        e = cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device);
     for (int v = 0; e == cudaSuccess && v < col_variants(p->M, p->periodic); v++) {
         e = col_tensor_maps(&p->cmaps[v], p->X, p->W, p->n, p->M, p->nrhs, v, p->periodic);
         if (e == cudaSuccess && p->Xs) e = col_tensor_maps(&p->cmaps_rc[v], p->Xs, p->W, p->n, p->M, p->nrhs, v);
@@ -834,14 +842,13 @@ tbs_status tbs_set_medium(tbs_plan_t p, const float *c, const float *alpha, doub
     cudaStream_t s = (cudaStream_t)stream;
     const size_t nn = (size_t)p->n * p->n;
     // the kernel that forms V also keeps copies of c and alpha (for gradients);
-    // what it cannot read (host memory, addresses off a float's boundary) is
-    // copied first
-    auto readable = [](const float *f) { return is_device_ptr(f) && (reinterpret_cast<uintptr_t>(f) & 3) == 0; };
-    if (!readable(c)) {
+    // what it cannot read (host memory, another device's, addresses off a
+    // float's boundary) is copied first
+    if (!kernel_may_use(p, c, sizeof(float))) {
         TBS_CK(cudaMemcpyAsync(p->c, c, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
         c = p->c;
     }
-    if (alpha && !readable(alpha)) {
+    if (alpha && !kernel_may_use(p, alpha, sizeof(float))) {
         TBS_CK(cudaMemcpyAsync(p->alpha, alpha, nn * sizeof(float), cudaMemcpyDeviceToDevice, s));
         alpha = p->alpha;
     }

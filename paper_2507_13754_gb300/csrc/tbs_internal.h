@@ -11,6 +11,13 @@ namespace tbs {
 // row starts 16-byte aligned and spans a multiple of 16 bytes (bulk copies).
 __host__ __device__ constexpr int ghat_stride(int M) { return M / 2 + 2; }
 
+// Whether a kernel on device `dev` may use memory that the runtime reports as
+// `type` on device `mem_dev`: managed memory, and that device's own.  (Another
+// device's memory reaches a plan by copies, which need no peer access.)
+inline bool kernel_reaches(cudaMemoryType type, int mem_dev, int dev) {
+    return type == cudaMemoryTypeManaged || (type == cudaMemoryTypeDevice && mem_dev == dev);
+}
+
 // Per right-hand-side solver state, updated by the stop test.
 struct RhsState {
     int done;        // 1 once the stop test has ended this RHS

@@ -3,7 +3,7 @@ not depend on how a call is launched."""
 import numpy as np
 import pytest
 
-from _helpers import gpu_plan, library
+from _helpers import gpu_plan, library, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +39,19 @@ def test_medium_at_any_address(off_c, off_a):
         p.close()
     assert np.abs(out[0]).max() > 0
     assert np.array_equal(out[0], out[1])
+
+
+# 2e-7: the bar of the other spectrum tests (one rounding to complex64).  At
+# k0 dx = 1e-27 the orders of the cell modes overflow FP64.
+@pytest.mark.parametrize("kh", [1e-27, 1e-18, 0.9e-9, 1.1e-9])
+@pytest.mark.parametrize("n", [9, 33])
+def test_ghat_at_any_fine_sampling(oracle_mod, n, kh):
+    import math
+    from paper_2507_13754_gb300 import tbs
+    c0, dx = 1500.0, 1e-3
+    f = kh * c0 / (2 * math.pi * dx)
+    plan = tbs.Plan(n, dx, f, c0)
+    gh = oracle_mod.ghat(n, plan.m, dx, oracle_mod.green_table(n, 2 * math.pi * f / c0, dx))
+    q = plan.m // 2 + 1
+    assert rel_l2(plan.ghat_quadrant(), gh[:q, :q]) < 2e-7
+    plan.close()

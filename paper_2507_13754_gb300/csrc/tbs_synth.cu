@@ -165,13 +165,13 @@ extern "C" tbs_status tbs_synthesize(const tbs_synth_freq *freqs, int32_t n_freq
     for (int c = 0; c < n_freq; c += SY_CHUNK) {
         SynthArgs a;
         memset(&a, 0, sizeof(a));
-        bool fast = t_max < 1e30;  // FP32 pairs hold t and f
+        bool fast = t_max < 1e30;  // FP32 pairs hold t and every f
         a.count = n_freq - c < SY_CHUNK ? n_freq - c : SY_CHUNK;
         for (int k = 0; k < a.count; k++) {
             const tbs_synth_freq &q = freqs[c + k];
             a.field[k] = (const float2 *)q.field;
             a.inv_dx[k] = 1.0 / q.dx;
-            fast = fast && fabs(q.freq_hz) * t_max < 65536.0;
+            fast = fast && fabs(q.freq_hz) < 1e30 && fabs(q.freq_hz) * t_max < 65536.0;
             a.f[k] = q.freq_hz;
             a.w[k] = (float)q.weight;
             a.n[k] = q.n;

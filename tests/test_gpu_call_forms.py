@@ -55,3 +55,19 @@ def test_ghat_at_any_fine_sampling(oracle_mod, n, kh):
     q = plan.m // 2 + 1
     assert rel_l2(plan.ghat_quadrant(), gh[:q, :q]) < 2e-7
     plan.close()
+
+
+def _phases(f, t0, dt, nt):
+    """exp(-2 pi i f t_j): the signal of a field of ones at weight 1."""
+    import torch
+    from paper_2507_13754_gb300 import tbs
+    ones = torch.ones((1, 2, 2), dtype=torch.complex64, device="cuda")
+    return tbs.synthesize([ones], [1.0], [f], [1.0], (0.0, 0.0), (0.0, 0.0), (1, 1), t0, dt, nt).cpu().numpy().ravel()
+
+
+# a phase rounded to FP32 (1.5e-8 cycles, 9.4e-8 rad) and the two components'
+# rounding (one unit in the last place each, 8.5e-8 together)
+@pytest.mark.parametrize("f,t0,dt,nt", [(1e39, 0.0, 0.0, 1), (-1e300, 0.0, 0.0, 3), (2.5e31, 1e-31, 1e-32, 5)])
+def test_synthesis_at_frequencies_beyond_fp32(f, t0, dt, nt):
+    t = t0 + np.arange(nt) * dt
+    assert np.abs(_phases(f, t0, dt, nt) - np.exp(-2j * np.pi * (f * t - np.rint(f * t)))).max() < 1.8e-7

@@ -458,8 +458,9 @@ tbs_status tbs_debug_set(tbs_plan_t plan, int32_t key, int64_t value);
  * Receivers: X = x0 + ix sx, Y = y0 + iy sy for 0 <= ix < nx, 0 <= iy < ny
  * [m].  Times: t_j = t0 + j dt, 0 <= j < n_t [s].
  * out: device complex64 [n_rhs][ny][nx][n_t] (caller-owned; overwritten).
- * Phases f_k t_j are reduced modulo 1 in FP64, or in FP32 pairs (about 2^-48 of
- * f t) where every |f t| < 2^16; samples and sums are FP32.
+ * Phases f_k t_j are reduced modulo 1 in FP64 and rounded to FP32, or kept as
+ * FP32 pairs (to 6e-10 cycles) where every |f t| < 2^16; samples and sums are
+ * FP32.
  * Asynchronous on `stream`; no device memory is allocated.
  * Errors: INVALID_ARG (NULL pointers, counts < 1, a bad frequency entry). */
 typedef struct tbs_synth_freq {

@@ -71,3 +71,14 @@ def _phases(f, t0, dt, nt):
 def test_synthesis_at_frequencies_beyond_fp32(f, t0, dt, nt):
     t = t0 + np.arange(nt) * dt
     assert np.abs(_phases(f, t0, dt, nt) - np.exp(-2j * np.pi * (f * t - np.rint(f * t)))).max() < 1.8e-7
+
+
+# |f t| to 2^16 cycles: the phase within 6e-10 cycles (4e-9 rad), sine and
+# cosine to one unit in the last place and one more rounding (9e-8 each)
+@pytest.mark.parametrize("f", [3.7, 5.123456e6])
+def test_synthesis_phase_error(f):
+    nt = 1 << 20
+    dt = 64729.13579 / f / nt
+    cyc = np.longdouble(f) * (np.arange(nt) * dt).astype(np.longdouble)
+    ref = np.exp(-2j * np.pi * (cyc - np.rint(cyc)).astype(np.float64))
+    assert np.abs(_phases(f, 0.0, dt, nt) - ref).max() < 1.33e-7

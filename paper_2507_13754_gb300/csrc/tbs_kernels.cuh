@@ -757,23 +757,40 @@ __device__ __forceinline__ bool group_sync_or(int id, int count, bool v) {
 // order: deterministic).  Results valid in the slot's thread 0.  Every call
 // passes one barrier over the slot (`sync`), after which all of the slot's
 // threads have made their calls.  red[k][w] holds slot warp w's sum of value k.
-template <int T, int K, class SYNC>
+// DF: double-float pairs within the warps too (row_sums, value for value), two
+// sums side by side in the halves of a warp.
+template <int T, int K, bool DF = false, class SYNC>
 __device__ __forceinline__ void slot_sums(const float (&x)[K], double (&out)[K], float2 (*red)[8], int t,
                                           const SYNC &sync) {
     static_assert(T >= 32 && T % 32 == 0 && T / 32 <= 8, "row slots of 1..8 warps");
-    float xs[K];
-#pragma unroll
-    for (int k = 0; k < K; k++) xs[k] = x[k];
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-#pragma unroll
-        for (int k = 0; k < K; k++) xs[k] += __shfl_xor_sync(0xffffffffu, xs[k], o);
-    }
-    DFloat v[K];
-#pragma unroll
-    for (int k = 0; k < K; k++) v[k] = DFloat{xs[k], 0.f};
     constexpr int WPR = T / 32;
     const int lane = t & 31, w = t >> 5;
+    DFloat v[K];
+    if constexpr (DF && K == 2) {
+        // the two sums side by side: lanes 0-15 take the first over, 16-31 the second
+        const bool up = (lane & 16) != 0;
+        const float other = __shfl_xor_sync(0xffffffffu, up ? x[0] : x[1], 16);
+        DFloat s = df_add(DFloat{up ? x[1] : x[0], 0.f}, DFloat{other, 0.f});
+#pragma unroll
+        for (int o = 8; o >= 1; o >>= 1)
+            s = df_add(s, DFloat{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)});
+        v[0] = s;
+        v[1] = DFloat{__shfl_xor_sync(0xffffffffu, s.hi, 16), __shfl_xor_sync(0xffffffffu, s.lo, 16)};
+    } else {
+#pragma unroll
+        for (int k = 0; k < K; k++) v[k] = DFloat{x[k], 0.f};
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) {
+#pragma unroll
+            for (int k = 0; k < K; k++) {
+                if constexpr (DF)
+                    v[k] = df_add(v[k], DFloat{__shfl_xor_sync(0xffffffffu, v[k].hi, o),
+                                               __shfl_xor_sync(0xffffffffu, v[k].lo, o)});
+                else
+                    v[k].hi += __shfl_xor_sync(0xffffffffu, v[k].hi, o);
+            }
+        }
+    }
     if (WPR > 1 && lane == 0) {
 #pragma unroll
         for (int k = 0; k < K; k++) red[k][w] = make_float2(v[k].hi, v[k].lo);
@@ -805,13 +822,14 @@ __device__ __forceinline__ void slot_sums(const float (&x)[K], double (&out)[K],
 // other row starts 8 bytes past a 16-byte boundary, so the copy begins one
 // element earlier (the row stands at `off` in the buffer) and ends on the next
 // boundary.  The elements beside the row are neighbours in the same plan
-// buffer, or its alignment padding, and are not used.
+// buffer, or its alignment padding, and are not used.  ODD = false: N is even.
+template <bool ODD = true>
 struct RowSpan {
     const float2 *p;
     unsigned bytes;
     int off;
     __device__ __forceinline__ RowSpan(const float2 *row, int n) {
-        off = (int)((reinterpret_cast<uintptr_t>(row) >> 3) & 1u);
+        off = ODD ? (int)((reinterpret_cast<uintptr_t>(row) >> 3) & 1u) : 0;
         p = row - off;
         bytes = (unsigned)(((n + off + 1) & ~1) * sizeof(float2));
     }
@@ -825,7 +843,11 @@ struct RowSpan {
 // the psi and V rows of the current row.  The next row's W is bulk-copied as
 // soon as the current one is in registers, and its psi and V rows once the
 // current epilogue has read them, so every copy has about a row's work to
-// land.  The arithmetic per row is exactly that of row_kernel<M, ROW_FWD>.
+// land.  The arithmetic per row is exactly that of row_kernel<M, ROW_FWD>,
+// except that for an even N the norms' sums within a warp are plain FP32.
+// ODD: N is odd: rows moved by RowSpan, the norms' sums in pairs throughout.
+// 3 x 999^2, 24 terms: 2502 us with one block per row, 2042 us here (2020 us
+// with FP32 sums, which lost up to 5e-10 of the norms).
 template <int M, int TH = 256>
 struct RowPCfg {
     static constexpr int E = 16, T = M / E;
@@ -839,7 +861,7 @@ struct RowPCfg {
     static_assert(LINE % 2 == 0 && M % 2 == 0 && HALF % 2 == 0, "16-byte aligned slot buffers");
 };
 
-template <int M, int TH>
+template <int M, int TH, bool ODD>
 __global__ void __launch_bounds__(RowPCfg<M, TH>::THREADS, 512 / TH)
 row_fwd_persistent_kernel(RowArgs a) {
     using C = RowPCfg<M, TH>;
@@ -893,7 +915,7 @@ row_fwd_persistent_kernel(RowArgs a) {
     };
     auto issue_pv = [&](int i) {  // slot thread 0
         const int r = i / n, y = i - r * n;
-        const RowSpan p(a.psi + (size_t)r * n * n + (size_t)y * n, n), v(a.V + (size_t)y * n, n);
+        const RowSpan<ODD> p(a.psi + (size_t)r * n * n + (size_t)y * n, n), v(a.V + (size_t)y * n, n);
         mbar_arrive_expect_tx(bar_pv, p.bytes + v.bytes);
         bulk_load(psi_s, p.p, p.bytes, bar_pv);
         bulk_load(v_s, v.p, v.bytes, bar_pv);
@@ -953,7 +975,8 @@ row_fwd_persistent_kernel(RowArgs a) {
             }
             return;
         }
-        const float2 *pr = psi_s + RowSpan(a.psi + row_sp, n).off, *vr = v_s + RowSpan(a.V + (size_t)y * n, n).off;
+        const float2 *pr = psi_s + RowSpan<ODD>(a.psi + row_sp, n).off;
+        const float2 *vr = v_s + RowSpan<ODD>(a.V + (size_t)y * n, n).off;
         // u -> psi += u, the norms' partial sums, V u; the N = M/2 grids (every
         // slot of the half row a grid point) skip the per-element bound
         auto epilogue = [&](auto full_c) {
@@ -979,7 +1002,7 @@ row_fwd_persistent_kernel(RowArgs a) {
                 }
             }
         };
-        if (n == M / 2)
+        if (!ODD && n == M / 2)
             epilogue(std::true_type{});
         else
             epilogue(std::false_type{});
@@ -990,11 +1013,11 @@ row_fwd_persistent_kernel(RowArgs a) {
         double su, sp, lu = 0.0, lp = 0.0;
         if (l1_here) {
             double o[4];
-            slot_sums<T, 4>({su_f, sp_f, lu_f, lp_f}, o, red, t, sync);
+            slot_sums<T, 4, ODD>({su_f, sp_f, lu_f, lp_f}, o, red, t, sync);
             su = o[0], sp = o[1], lu = o[2], lp = o[3];
         } else {
             double o[2];
-            slot_sums<T, 2>({su_f, sp_f}, o, red, t, sync);
+            slot_sums<T, 2, ODD>({su_f, sp_f}, o, red, t, sync);
             su = o[0], sp = o[1];
         }
         if (t == 0) {
@@ -1075,7 +1098,7 @@ row_adj_persistent_kernel(RowArgs a) {
     };
     auto issue_q = [&](int i) {  // slot thread 0
         const int r = i / n, y = i - r * n;
-        const RowSpan q(a.Q + (size_t)i * n, n), u(Uj + r * a.u_rhs + (size_t)y * n, n), g(a.src + (size_t)i * n, n);
+        const RowSpan<> q(a.Q + (size_t)i * n, n), u(Uj + r * a.u_rhs + (size_t)y * n, n), g(a.src + (size_t)i * n, n);
         mbar_arrive_expect_tx(bar_q, q.bytes + u.bytes);
         bulk_load(q_s, q.p, q.bytes, bar_q);
         bulk_load(u_s, u.p, u.bytes, bar_q);
@@ -1121,7 +1144,7 @@ row_adj_persistent_kernel(RowArgs a) {
         }
         float2 *Q = a.Q + (size_t)i * n;
         const float2 *g = a.src + (size_t)i * n, *V = a.V + (size_t)y * n;
-        const float2 *qr = q_s + RowSpan(Q, n).off, *ur = u_s + RowSpan(Uj + rhs * a.u_rhs + (size_t)y * n, n).off;
+        const float2 *qr = q_s + RowSpan<>(Q, n).off, *ur = u_s + RowSpan<>(Uj + rhs * a.u_rhs + (size_t)y * n, n).off;
         constexpr int CH = 4;  // a batch's loads are issued together
 #pragma unroll
         for (int m0 = 0; m0 < E / 2; m0 += CH) {
@@ -2230,7 +2253,8 @@ static cudaError_t row_launch_th(int nrhs, const RowArgs &b, cudaStream_t s) {
     if constexpr ((KIND == ROW_FWD || KIND == ROW_ADJ) && M >= 512) {
         if (b.num_sms > 0) {
             if constexpr (KIND == ROW_FWD)
-                return persistent_row<row_fwd_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
+                return b.n & 1 ? persistent_row<row_fwd_persistent_kernel<M, TH, true>, RowPCfg<M, TH>>(nrhs, b, s)
+                               : persistent_row<row_fwd_persistent_kernel<M, TH, false>, RowPCfg<M, TH>>(nrhs, b, s);
             else
                 return persistent_row<row_adj_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
         }
@@ -2510,7 +2534,8 @@ static cudaError_t row_attr() {
     set(row_kernel<M, ROW_EPSK, TH>, b);
     set(row_kernel<M, ROW_OUT, TH>, b);
     if constexpr (M >= 512) {
-        set(row_fwd_persistent_kernel<M, TH>, (int)RowPCfg<M, TH>::SMEM);
+        set(row_fwd_persistent_kernel<M, TH, false>, (int)RowPCfg<M, TH>::SMEM);
+        set(row_fwd_persistent_kernel<M, TH, true>, (int)RowPCfg<M, TH>::SMEM);
         set(row_adj_persistent_kernel<M, TH>, (int)RowPCfg<M, TH>::SMEM);
         set(row_eps_persistent_kernel<M, false, TH>, (int)RowECfg<M, TH>::SMEM);
         set(row_eps_persistent_kernel<M, true, TH>, (int)RowECfg<M, TH>::SMEM);

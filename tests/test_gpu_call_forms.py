@@ -3,7 +3,7 @@ not depend on how a call is launched."""
 import numpy as np
 import pytest
 
-from _helpers import gpu_plan, library, rel_l2
+from _helpers import gpu_plan, gpu_solve, library, rel_l2
 
 pytestmark = pytest.mark.gpu
 
@@ -82,3 +82,25 @@ def test_synthesis_phase_error(f):
     cyc = np.longdouble(f) * (np.arange(nt) * dt).astype(np.longdouble)
     ref = np.exp(-2j * np.pi * (cyc - np.rint(cyc)).astype(np.float64))
     assert np.abs(_phases(f, 0.0, dt, nt) - ref).max() < 1.33e-7
+
+
+@pytest.mark.parametrize("n", [257, 511, 513, 1025])
+def test_norms_of_odd_grids(n):
+    """psi_norm against FP64 sums of each thread's FP32 sum of squares (formed
+    here from the field it belongs to): the sums across threads carry double-
+    float pairs, 48 bits.  1e-10 leaves room for a thread's sum that this
+    emulation rounds twice (6e-8 of one of n^2 / 8 sums)."""
+    from paper_2507_13754_gb300 import workloads as W
+    w = W.random_medium(n, seed=72)
+    w.max_terms, w.tol = 4, 0.0
+    psi, info, plan = gpu_solve(w)
+    T = plan.m // 16
+    x = np.zeros((n, 8 * T, 2))
+    x[:, :n, 0], x[:, :n, 1] = psi[0].real, psi[0].imag
+    x = x.reshape(n, 8, T, 2)
+    s = np.zeros((n, T), np.float32)
+    for m in range(8):
+        s = (x[:, m, :, 1] ** 2 + s).astype(np.float32)
+        s = (x[:, m, :, 0] ** 2 + s).astype(np.float32)
+    assert abs(info[0]["psi_norm"] / np.sqrt(s.sum(dtype=np.float64)) - 1) < 1e-10
+    plan.close()

@@ -330,6 +330,7 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     sa.div_grace = p->d.div_grace;
     sa.div_window = p->d.div_window;
     sa.div_factor = p->d.div_factor;
+    sa.sums = stop_sums(p->M);
     sa.loop_ctl = nullptr;
     sa.loop = 0;
     // in the term loop the row pass and the stop kernel are programmatic

@@ -27,7 +27,14 @@ namespace tbs {
 __global__ void __launch_bounds__(256) stop_kernel(StopArgs a) {
     grid_dep_wait();
     const int rhs = blockIdx.x;
-    if (!a.st[rhs].done) reduce_and_decide(a, rhs);
+    if (!a.st[rhs].done) {
+        if (a.sums == 32)
+            reduce_and_decide<32>(a, rhs);
+        else if (a.sums == 128)
+            reduce_and_decide<128>(a, rhs);
+        else
+            reduce_and_decide<256>(a, rhs);
+    }
     if (a.loop_ctl && threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(a.loop_ctl, 1) == (int)gridDim.x - 1) {

@@ -321,39 +321,48 @@ __device__ __forceinline__ void stop_decide(const StopArgs &a, int rhs, double s
     s->done = done;
 }
 
-// Fixed-order FP64 reduction of the row partials of one RHS by a block of
-// whole warps (per-thread strided sums, shuffle trees within and then across
-// the warps), then the stop decision in thread 0.
+// FP64 reduction of the row partials of one RHS by the first SUMS threads of a
+// block, then the stop decision in thread 0.  Partial y goes to sum y mod
+// SUMS, the sums through shuffle trees within and then across the warps.
+// SUMS follows M alone (stop_sums), so a term's records are the same bits
+// whichever kernel and tile shape makes its test.
+template <int SUMS>
 __device__ __forceinline__ void reduce_and_decide(const StopArgs &a, int rhs) {
-    __shared__ double2 rw[32];
-    double su = 0.0, sp = 0.0;
+    constexpr int WARPS = SUMS / 32;
+    static_assert(SUMS % 32 == 0 && WARPS <= 8, "whole warps");
+    __shared__ double2 rw[8];
     const double2 *part = a.part + (size_t)rhs * a.n;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double su = 0.0, sp = 0.0;
+    if (warp < WARPS) {
 #pragma unroll 8
-    for (int y = threadIdx.x; y < a.n; y += blockDim.x) {
-        const double2 q = __ldcg(part + y);
-        su += q.x;
-        sp += q.y;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        su += __shfl_xor_sync(0xffffffffu, su, o);
-        sp += __shfl_xor_sync(0xffffffffu, sp, o);
-    }
-    if (lane == 0) rw[warp] = make_double2(su, sp);
-    __syncthreads();
-    if (warp == 0) {
-        const double2 q = lane < warps ? rw[lane] : make_double2(0.0, 0.0);
-        su = q.x;
-        sp = q.y;
+        for (int y = threadIdx.x; y < a.n; y += SUMS) {
+            const double2 q = __ldcg(part + y);
+            su += q.x;
+            sp += q.y;
+        }
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) {
             su += __shfl_xor_sync(0xffffffffu, su, o);
             sp += __shfl_xor_sync(0xffffffffu, sp, o);
         }
+        if (WARPS > 1 && lane == 0) rw[warp] = make_double2(su, sp);
+    }
+    if (WARPS > 1) __syncthreads();
+    if (warp == 0) {
+        if (WARPS > 1) {
+            const double2 q = rw[lane & (WARPS - 1)];
+            su = q.x;
+            sp = q.y;
+#pragma unroll
+            for (int o = WARPS / 2; o >= 1; o >>= 1) {
+                su += __shfl_xor_sync(0xffffffffu, su, o);
+                sp += __shfl_xor_sync(0xffffffffu, sp, o);
+            }
+        }
         if (lane == 0) stop_decide(a, rhs, su, sp);
     }
-    __syncthreads();  // rw may be written again
+    __syncthreads();  // rw may be written again, every thread reads the next flag
 }
 
 // The stop test inside a column pass: block gridDim.x - 1 - r decides for RHS
@@ -363,10 +372,14 @@ __device__ __forceinline__ void reduce_and_decide(const StopArgs &a, int rhs) {
 // serial chain (the partials' loads, FP64 sums, two square roots and a
 // division: 6 to 10 us as a kernel of its own at N = 256 .. 4096) that nothing
 // of the column pass needs; the last blocks are those with the fewest tiles.
+template <int M, int THREADS>
 __device__ __forceinline__ void col_stop(const StopArgs &a, int nrhs) {
-    if (!a.st) return;
-    for (int r = (int)gridDim.x - 1 - (int)blockIdx.x; r < nrhs; r += gridDim.x)
-        if (__ldcg(&a.st[r].done) == 0) reduce_and_decide(a, r);
+    if constexpr (M >= 128) {
+        static_assert(THREADS % 32 == 0 && THREADS >= stop_sums(M), "the sums' threads");
+        if (!a.st) return;
+        for (int r = (int)gridDim.x - 1 - (int)blockIdx.x; r < nrhs; r += gridDim.x)
+            if (__ldcg(&a.st[r].done) == 0) reduce_and_decide<stop_sums(M)>(a, r);
+    }
 }
 
 // A forward row pass leaves each RHS's flag as it stood before this pass: the
@@ -1651,7 +1664,7 @@ col_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid_cons
         __syncthreads();
         issue(i, 0);
     }
-    col_stop(a.stop, a.nrhs);
+    col_stop<M, C::THREADS>(a.stop, a.nrhs);
     int prev = -1;  // tile whose output rows wait in the other stage
     for (int buf = 0; i < total; buf ^= 1) {
         const int inext = next_active(i + gridDim.x);
@@ -1844,7 +1857,7 @@ col_pipe_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid
         load_ghat(cur);
         if (nx1 < total) load_rows(nx1, D1, &bars[1]);
     }
-    col_stop(a.stop, a.nrhs);
+    col_stop<M, C::THREADS>(a.stop, a.nrhs);
     fl0 = cur < total;
     flg = !C::PER && cur < total;
     fl1 = nx1 < total;
@@ -2112,7 +2125,7 @@ col_compact_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __g
     const Lines<2, true> sm{lines + 2 * cg * C::LSTRIDE, C::LSTRIDE};
     int cur = next_active(blockIdx.x);
     if (threadIdx.x == 0 && cur < total) load_rows(cur);
-    col_stop(a.stop, a.nrhs);
+    col_stop<M, C::THREADS>(a.stop, a.nrhs);
     unsigned ph = 0u;  // both barriers complete once per tile
     while (cur < total) {
         const int nxt = next_active(cur + gridDim.x);

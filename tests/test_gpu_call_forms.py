@@ -104,3 +104,41 @@ def test_norms_of_odd_grids(n):
         s = (x[:, m, :, 0] ** 2 + s).astype(np.float32)
     assert abs(info[0]["psi_norm"] / np.sqrt(s.sum(dtype=np.float64)) - 1) < 1e-10
     plan.close()
+
+
+@pytest.mark.parametrize("n,n_rhs", [(64, 16), (128, 24), (256, 24), (512, 8), (1024, 8)])
+def test_records_do_not_depend_on_the_launch(n, n_rhs):
+    """The same bits whether a term's stop test is made by a kernel of its own
+    (the last of max_terms, launched from the host), inside a column pass of
+    any tile shape (a term that ends a series to a residual), with the RHS
+    alone in its plan or among others.  The periodic grid's Green's function
+    decays: the rows' sums span so many binades that another order of theirs
+    rounds otherwise."""
+    import math
+    import torch
+    from paper_2507_13754_gb300 import tbs, workloads as W
+    w = W.random_medium(n, seed=71, n_rhs=n_rhs)
+    k0 = 2 * math.pi * w.f / w.c0
+
+    def solve(amp, max_terms, tol, variant=0, **kw):
+        p = tbs.Plan(n, w.dx, w.f, w.c0, n_rhs=len(amp), max_terms=max_terms, tol=tol, periodic=True,
+                     div_window=1 << 30, div_factor=math.inf, **kw)
+        p.set_potential(torch.full((n, n), 0.05 * k0 * k0, dtype=torch.complex64, device="cuda"))
+        p.set_sources(w.src_ix, w.src_iy, amp)
+        variants = tbs.tbs_col_variants(p.handle)
+        tbs.tbs_set_col_variant(p.handle, variant % variants)
+        info = tbs.Plan.info_dicts(p.solve()[1])
+        p.close()
+        return [(i["terms"], i["residual"], i["term_norm_max"], i["psi_norm"]) for i in info], variants
+
+    ref, variants = solve(w.src_amp, 3, 0.0, use_graph=False)
+    tol = max(r[1] for r in ref) * (1 + 1e-6)
+    assert all(r[0] == 3 for r in ref) and 0 < tol < 1
+    for v in range(variants):
+        got, _ = solve(w.src_amp, 40, tol, v)
+        ended = [r for r in range(n_rhs) if got[r][0] == 3]
+        assert ended
+        assert [got[r] for r in ended] == [ref[r] for r in ended], v
+    for r in range(0, n_rhs, 3):
+        one, _ = solve(w.src_amp[r:r + 1], 40, ref[r][1] * (1 + 1e-6))
+        assert one[0] == ref[r], r

@@ -8,10 +8,10 @@
 //     row pass on S  ->  { column pass + stop test, row pass } while active
 //
 // and the host never waits between terms.  tbs_solve captures it once into a
-// CUDA graph (on a plan-owned stream) and replays it: the loop is a WHILE
-// conditional node whose condition the stop test sets, so the graph runs the
-// terms the slowest RHS needs (in bodies of several; launches past an RHS's stop
-// return at once).  Without a graph (timing,
+// CUDA graph (on a plan-owned stream) and replays it: the first terms, then a
+// WHILE conditional node whose condition the stop test sets, so the graph runs
+// the terms the slowest RHS needs (in bodies of several, term_loop; launches past
+// an RHS's stop return at once).  Without a graph (timing,
 // TBS_FLAG_NO_GRAPH) the loop is unrolled max_terms times on the stream and
 // launches after every RHS has stopped return at once.  Each launch checks
 // its RHS's device flag, so an RHS that stopped early does no further work.
@@ -239,14 +239,14 @@ cudaError_t timed_col(tbs_plan_s *p, bool cj, const ColArgs &a, cudaStream_t s) 
     return e;
 }
 
-// A condition for a WHILE node in the graph being captured on s; each
-// launch of the graph resets it to 1.
-tbs_status loop_condition(cudaStream_t s, cudaGraphConditionalHandle *h) {
+// A condition for a WHILE node in the graph being captured on s; each launch
+// of the graph resets it to `initial`.
+tbs_status loop_condition(cudaStream_t s, cudaGraphConditionalHandle *h, unsigned initial) {
     cudaStreamCaptureStatus cs;
     cudaGraph_t g = nullptr;
     TBS_CK(cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, nullptr, nullptr, nullptr));
     if (cs != cudaStreamCaptureStatusActive) return fail(TBS_ERR_STATE, "graph loop outside a stream capture");
-    TBS_CK(cudaGraphConditionalHandleCreate(h, g, 1, cudaGraphCondAssignDefault));
+    TBS_CK(cudaGraphConditionalHandleCreate(h, g, initial, cudaGraphCondAssignDefault));
     return TBS_OK;
 }
 
@@ -354,39 +354,35 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     // (the medium and sources may change between solves of a plan)
     if (rk == ROW_EPS) TBS_CK(launch_row_flags(p->n, p->nrhs, p->V, p->S, p->vflag, p->sflag, s));
     if (graph_loop) {
-        // The body runs `body` terms; each kernel reads its RHS's term index
-        // from the RHS state and returns at once for an RHS that has stopped.
-        // The last stop test of the body sets the condition.  An iteration
-        // costs 7 us beyond the launches it holds, a term's launches after the
-        // stop about 4 us, so to a residual the body holds 8 terms (4 -> 8: a
-        // term at N = 64 / 256 / 1024 1.0 / 1.0 / 1.2 us less), and a fixed number
-        // of terms is split into equal bodies of at most 16.
-        const int bodies = (p->d.max_terms + 15) / 16;
-        const int body = p->d.tol > 0 ? 8 : (p->d.max_terms + bodies - 1) / bodies;
-        cudaGraphConditionalHandle h;
-        tbs_status st = loop_condition(s, &h);
-        if (st != TBS_OK) return st;
-        ra.term = -1;
-        sa.term = -1;
-        st = capture_while(p, s, h, [&](cudaStream_t b) {
+        // Each kernel reads its RHS's term index from the RHS state and returns
+        // at once for an RHS that has stopped.  The stop test at the end of the
+        // lead and of each body sets the loop's condition.
+        ca.gate.mode = ra.gate.mode = GATE_FWD;
+        ra.term = sa.term = -1;
+        auto terms = [&](cudaStream_t b, int count, const cudaGraphConditionalHandle *h) {
             cudaError_t e = cudaSuccess;
-            for (int k = 0; k < body && e == cudaSuccess; k++) {
+            for (int k = 0; k < count && e == cudaSuccess; k++) {
                 ColArgs ck = ca;
                 ck.early = beside;
                 ck.pdl = k > 0 && (early || !fused);  // follows a row pass (or a stop test)
                 if (k > 0 && fused) ck.stop = sa, ck.gate.before_row = 1;
                 StopArgs sk = sa;
-                sk.loop = h;
-                sk.loop_ctl = k == body - 1 ? p->err + 1 : nullptr;
+                if (k == count - 1 && h) sk.loop = *h, sk.loop_ctl = p->err + 1;
                 e = launch_col(p->M, p->nrhs, false, ck, &p->cmaps[p->col_variant], p->col_variant, b);
                 if (e == cudaSuccess) e = launch_row(rk, p->M, p->nrhs, ra, b);
                 // before the condition is evaluated; earlier terms' tests are
                 // the next column pass's
-                if (e == cudaSuccess && (sk.loop_ctl || !fused)) e = launch_stop(p->nrhs, sk, b);
+                if (e == cudaSuccess && (k == count - 1 || !fused)) e = launch_stop(p->nrhs, sk, b);
             }
             return e;
-        });
-        if (st != TBS_OK) return st;
+        };
+        const TermLoop l = term_loop(p->d.max_terms, p->d.tol > 0);
+        cudaGraphConditionalHandle loop;
+        tbs_status st;
+        if (l.body && (st = loop_condition(s, &loop, l.lead ? 0 : 1)) != TBS_OK) return st;
+        TBS_CK(terms(s, l.lead, l.body ? &loop : nullptr));
+        if (l.body && (st = capture_while(p, s, loop, [&](cudaStream_t b) { return terms(b, l.body, &loop); })) != TBS_OK)
+            return st;
     } else {
         for (int t = 0; t < p->d.max_terms; t++) {
             if (t > 0 && fused) ca.stop = sa, ca.gate.before_row = 1;  // the test of term t - 1
@@ -450,7 +446,7 @@ tbs_status enqueue_adjoint(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     if (graph_loop) {
         int *jdev = p->err + 3;
         cudaGraphConditionalHandle h;
-        tbs_status st = loop_condition(s, &h);
+        tbs_status st = loop_condition(s, &h, 1);
         if (st != TBS_OK) return st;
         TBS_CK(launch_adj_loop(p->nrhs, p->state, jdev, h, true, 0, s));
         ra.term = -1;

@@ -33,6 +33,37 @@ struct RhsState {
     int pad_;
 };
 
+// How a solve's graph holds its terms: `lead` terms outright, then a WHILE node
+// of `body` terms per iteration (0: no node).  The node costs 7 us (N = 64) to
+// 14 us (N >= 700) per iteration beyond its launches, also when it is not
+// entered, a term's launches after the stop 3 to 7 us.
+//  * to a residual: 4 terms, then equal bodies of at most 8.  With 8-term
+//    bodies alone a series of one term paid for 8: 111 -> 88 us at N = 700,
+//    122 -> 99 us at N = 1024 (101 us with bodies of 4).  Longer series end in
+//    another place of a body: at N = 700, 8 / 12 / 16 / 20 terms 286 / 455 / 549
+//    / 719 -> 322 / 415 / 584 / 677 us (338 / 491 / 644 / 795 us with bodies of 4).
+//  * a fixed number of terms: the WHILE alone, with the body (at most 16) of
+//    the least cost at 7 us an iteration and 4 us an empty term.
+struct TermLoop {
+    int lead, body;
+};
+inline TermLoop term_loop(int max_terms, bool to_residual) {
+    TermLoop l = {0, 0};
+    if (to_residual) {
+        l.lead = max_terms <= 6 ? max_terms : 4;
+        const int rest = max_terms - l.lead, iterations = (rest + 7) / 8;
+        if (iterations > 0) l.body = (rest + iterations - 1) / iterations;
+        return l;
+    }
+    int best = 0;
+    for (int b = max_terms < 16 ? max_terms : 16; b >= 1; b--) {
+        const int iterations = (max_terms + b - 1) / b;
+        const int cost = 7 * iterations + 4 * (iterations * b - max_terms);
+        if (l.body == 0 || cost < best) l.body = b, best = cost;
+    }
+    return l;
+}
+
 // Which right-hand sides a launch works on.
 enum GateMode { GATE_ALL = 0, GATE_FWD = 1, GATE_ADJ = 2 };
 struct Gate {

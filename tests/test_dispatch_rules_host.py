@@ -31,3 +31,30 @@ def test_kernels_get_their_own_device_memory_only(tmp_path):
         for (int m = 0; m < 2; m++) printf("%d ", (int)kernel_reaches(t[k], m, 1));
     ''')
     assert got == list("00000111")
+
+
+def test_graph_loops_launch_little_beyond_a_series(tmp_path):
+    """Terms launched for a series of T terms.  To a residual: at most 6 within
+    4, at most 7 beyond T, none beyond max_terms up to 12.  A fixed number: no
+    body of at most 16 has fewer iterations (7 us) and empty terms (4 us)."""
+    v = iter(_run(tmp_path, r'''
+    for (int m = 1; m <= 300; m++)
+        for (int r = 0; r < 2; r++) {
+            const TermLoop l = term_loop(m, r != 0);
+            printf("%d %d ", l.lead, l.body);
+        }
+    '''))
+    for m in range(1, 301):
+        for residual in (False, True):
+            lead, body = int(next(v)), int(next(v))
+            assert lead <= m and (lead == m) == (body == 0)
+
+            def launched(t):
+                return lead + (-(-max(t - lead, 0) // body) * body if body else 0)
+
+            if residual:
+                assert lead <= 6 and all(t <= launched(t) <= t + 7 for t in range(1, m + 1))
+                assert m > 12 or launched(m) == m
+            else:
+                cost = [7 * -(-m // b) + 4 * (-(-m // b) * b - m) for b in range(1, min(m, 16) + 1)]
+                assert lead == 0 and 7 * (launched(m) // body) + 4 * (launched(m) - m) == min(cost)

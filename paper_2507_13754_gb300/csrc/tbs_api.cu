@@ -431,7 +431,8 @@ tbs_status enqueue_outputs(tbs_plan_s *p, float *psi, tbs_solve_info *info, bool
 // Reverse sweep of the truncated series (the plan's stored terms u_j):
 // ubar_{T-1} = g; for j = T-2 .. 0: lambda = G^H ubar_{j+1}, Q += conj(lambda)
 // u_j, ubar_j = g + conj(V) lambda, with T the RHS's own term count.  In a
-// graph the steps are a WHILE node whose counter starts at max_r T_r - 2.
+// graph the steps are a WHILE node whose counter starts at max_r T_r - 2
+// (reverse_loop).
 tbs_status enqueue_adjoint(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     const size_t nn = (size_t)p->n * p->n;
     TBS_CK(cudaMemsetAsync(p->Q, 0, sizeof(float2) * p->nrhs * nn, s));
@@ -445,25 +446,29 @@ tbs_status enqueue_adjoint(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     const bool early = early_columns(p);
     if (graph_loop) {
         int *jdev = p->err + 3;
-        cudaGraphConditionalHandle h;
-        tbs_status st = loop_condition(s, &h, 1);
-        if (st != TBS_OK) return st;
-        TBS_CK(launch_adj_loop(p->nrhs, p->state, jdev, h, true, 0, s));
         ra.term = -1;
         ra.gate.j = ca.gate.j = -1;
         ra.gate.jdev = ca.gate.jdev = jdev;
-        return capture_while(p, s, h, [&](cudaStream_t b) {
-            // several steps per iteration, as in the forward loop; those below
-            // step 0 return at once
-            constexpr int STEPS = 8;
+        auto sweep = [&](cudaStream_t b, int count) {  // those below step 0 return at once
             cudaError_t e = cudaSuccess;
-            for (int k = 0; k < STEPS && e == cudaSuccess; k++) {
+            for (int k = 0; k < count && e == cudaSuccess; k++) {
                 ra.gate.back = ca.gate.back = k;
                 ca.pdl = k > 0 && early;
                 e = launch_col(p->M, p->nrhs, true, ca, &p->cmaps[p->col_variant], p->col_variant, b);
                 if (e == cudaSuccess) e = launch_row(ROW_ADJ, p->M, p->nrhs, ra, b);
             }
-            return e == cudaSuccess ? launch_adj_loop(p->nrhs, p->state, jdev, h, false, STEPS, b) : e;
+            return e;
+        };
+        const ReverseLoop l = reverse_loop(p->d.max_terms);
+        cudaGraphConditionalHandle h;
+        tbs_status st;
+        if (l.body && (st = loop_condition(s, &h, 0)) != TBS_OK) return st;
+        TBS_CK(launch_adj_loop(p->nrhs, p->state, jdev, l.body ? &h : nullptr, 0, s));
+        TBS_CK(sweep(s, l.lead));
+        if (!l.body) return TBS_OK;
+        return capture_while(p, s, h, [&](cudaStream_t b) {
+            const cudaError_t e = sweep(b, l.body);
+            return e == cudaSuccess ? launch_adj_loop(p->nrhs, p->state, jdev, &h, l.body, b) : e;
         });
     }
     for (int j = p->d.max_terms - 2; j >= 0; j--) {

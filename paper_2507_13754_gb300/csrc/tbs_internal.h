@@ -64,6 +64,21 @@ inline TermLoop term_loop(int max_terms, bool to_residual) {
     return l;
 }
 
+// The reverse sweep's steps likewise: `lead` steps outright where max_terms allows
+// no more than 6, else a WHILE of equal bodies of at most 4.  Sweeps of 2, 4, 8 and
+// 16 steps at N = 300 with 4 RHS: 100, 158, 280, 532 us with one step per
+// iteration, 124, 163, 241, 442 us with 8 (a sweep of one step paid for 8),
+// 102, 140, 245, 445 us with 4.
+struct ReverseLoop {
+    int lead, body;
+};
+inline ReverseLoop reverse_loop(int max_terms) {
+    const int steps = max_terms - 1, iterations = (steps + 3) / 4;
+    ReverseLoop l = {steps, 0};
+    if (steps > 6) l.lead = 0, l.body = (steps + iterations - 1) / iterations;
+    return l;
+}
+
 // Which right-hand sides a launch works on.
 enum GateMode { GATE_ALL = 0, GATE_FWD = 1, GATE_ADJ = 2 };
 struct Gate {
@@ -211,9 +226,9 @@ const char *col_variant_name(int M, bool periodic, int variant);
 cudaError_t col_tensor_maps(ColMaps *maps, const float2 *X, const float2 *W, int n, int M, int nrhs, int variant,
                             bool periodic = false);
 cudaError_t launch_stop(int nrhs, const StopArgs &a, cudaStream_t s);
-// Adjoint graph loop control (one thread): with init, *j = max_r terms_r - 2,
-// else *j -= steps; then the WHILE condition is set to (*j >= 0).
-cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphConditionalHandle h, bool init, int steps,
+// Adjoint graph loop control (one thread): *j = max_r terms_r - 2 (steps 0) or
+// *j -= steps; then, with h given, the WHILE condition is set to (*j >= 0).
+cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, const cudaGraphConditionalHandle *h, int steps,
                             cudaStream_t s);
 // A solve's outputs: its records to info (8-byte aligned device memory) and, in
 // the same kernel, psi copied to out (out null: records only; out 16-byte

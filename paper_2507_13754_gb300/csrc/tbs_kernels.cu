@@ -58,10 +58,10 @@ struct InfoOut {  // layout of tbs_solve_info
     double psi_norm;
 };
 
-__global__ void adj_loop_kernel(int nrhs, const RhsState *st, int *jdev, cudaGraphConditionalHandle h, int init,
+__global__ void adj_loop_kernel(int nrhs, const RhsState *st, int *jdev, int loop, cudaGraphConditionalHandle h,
                                 int steps) {
     int j;
-    if (init) {
+    if (steps == 0) {
         int tmax = 0;
         for (int r = 0; r < nrhs; r++) tmax = max(tmax, st[r].terms);
         j = tmax - 2;
@@ -69,7 +69,7 @@ __global__ void adj_loop_kernel(int nrhs, const RhsState *st, int *jdev, cudaGra
         j = *jdev - steps;
     }
     *jdev = j;
-    cudaGraphSetConditional(h, j >= 0 ? 1u : 0u);
+    if (loop) cudaGraphSetConditional(h, j >= 0 ? 1u : 0u);
 }
 
 // The records (one thread per RHS of the first blocks) and the copy of psi,
@@ -344,9 +344,9 @@ cudaError_t launch_stop(int nrhs, const StopArgs &a, cudaStream_t s) {
     return launch_k(stop_kernel, dim3(nrhs), dim3(256), 0, s, a.pdl != 0, a);
 }
 
-cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, cudaGraphConditionalHandle h, bool init, int steps,
+cudaError_t launch_adj_loop(int nrhs, const RhsState *st, int *j, const cudaGraphConditionalHandle *h, int steps,
                             cudaStream_t s) {
-    adj_loop_kernel<<<1, 1, 0, s>>>(nrhs, st, j, h, init ? 1 : 0, steps);
+    adj_loop_kernel<<<1, 1, 0, s>>>(nrhs, st, j, h != nullptr, h ? *h : 0, steps);
     return cudaGetLastError();
 }
 

@@ -58,3 +58,21 @@ def test_graph_loops_launch_little_beyond_a_series(tmp_path):
             else:
                 cost = [7 * -(-m // b) + 4 * (-(-m // b) * b - m) for b in range(1, min(m, 16) + 1)]
                 assert lead == 0 and 7 * (launched(m) // body) + 4 * (launched(m) - m) == min(cost)
+
+
+def test_reverse_loops_launch_few_empty_steps(tmp_path):
+    """A sweep of S steps: none launched beyond max_terms - 1 up to 6 of them,
+    at most 3 empty ones in a loop."""
+    v = iter(_run(tmp_path, r'''
+    for (int m = 1; m <= 300; m++) {
+        const ReverseLoop l = reverse_loop(m);
+        printf("%d %d ", l.lead, l.body);
+    }
+    '''))
+    for m in range(1, 301):
+        lead, body = int(next(v)), int(next(v))
+        if m <= 7:
+            assert (lead, body) == (m - 1, 0)
+        else:
+            assert lead == 0 and 3 <= body <= 4
+            assert -(-(m - 1) // body) == -(-(m - 1) // 4)  # as few iterations as bodies of 4

@@ -384,10 +384,15 @@ __device__ __forceinline__ void col_stop(const StopArgs &a, int nrhs) {
 
 // A forward row pass leaves each RHS's flag as it stood before this pass: the
 // column pass that follows changes `done` while its blocks run, so they read
-// this copy instead (every thread of a launch sees one value).
+// this copy instead (every thread of a launch sees one value).  In the
+// persistent passes thread i of the grid copies RHS i's; with one block per row
+// an RHS's first block does.  (One thread for all of them, a load and a store
+// each, outlasted the pass: 10 terms of 1024 RHS at N = 32 609 -> 514 us, of
+// 65535 RHS at N = 16 29.5 -> 16.4 ms.)
 __device__ __forceinline__ void mark_before_row(const RowArgs &a) {
-    if (a.gate.mode == GATE_FWD && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
-        for (int r = 0; r < a.nrhs; r++) a.gate.st[r].before_row = a.gate.st[r].done;
+    if (a.gate.mode == GATE_FWD)
+        for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < a.nrhs; r += gridDim.x * blockDim.x)
+            a.gate.st[r].before_row = a.gate.st[r].done;
 }
 
 // Optional phase timers for experiments (compiled out unless defined).
@@ -469,7 +474,9 @@ row_kernel(RowArgs a) {
         }
     }
     grid_dep_launch();  // the next kernel may be scheduled once every row block runs
-    if constexpr (KIND == ROW_FWD || KIND == ROW_EPS || KIND == ROW_EPSK) mark_before_row(a);
+    if constexpr (KIND == ROW_FWD || KIND == ROW_EPS || KIND == ROW_EPSK)
+        if (a.gate.mode == GATE_FWD && blockIdx.x == 0 && threadIdx.x == 0)
+            a.gate.st[rhs].before_row = a.gate.st[rhs].done;
     if constexpr (KIND == ROW_SRC) {  // a solve or G application begins: zero its state and error words
         if (blockIdx.x == 0 && blockIdx.y == 0) {
             for (int i = threadIdx.x; i < a.clear_words; i += C::THREADS) reinterpret_cast<int *>(a.clear)[i] = 0;

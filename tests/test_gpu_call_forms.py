@@ -142,3 +142,24 @@ def test_records_do_not_depend_on_the_launch(n, n_rhs):
     for r in range(0, n_rhs, 3):
         one, _ = solve(w.src_amp[r:r + 1], 40, ref[r][1] * (1 + 1e-6))
         assert one[0] == ref[r], r
+
+
+@pytest.mark.parametrize("n,n_rhs", [(20, 700), (64, 300), (140, 70), (260, 40)])
+def test_many_rhs_stop_on_their_own(n, n_rhs):
+    """Hundreds of RHS that stop after different numbers of terms: each has the
+    field and records that it has in a plan of its own few."""
+    from paper_2507_13754_gb300 import workloads as W
+    w = W.random_medium(n, seed=73, n_rhs=n_rhs)
+    w.alpha *= np.float32(1500.0 / n)
+    w.src_amp[::3, 1:] = 0
+    w.src_amp[5] = 0
+    psi, info, plan = gpu_solve(w, max_terms=40, tol=1e-4)
+    plan.close()
+    assert len({i["terms"] for i in info}) > 1
+    amp = w.src_amp
+    for r0 in range(0, n_rhs, 9):
+        w.src_amp = amp[r0:r0 + 5]
+        some, some_info, p = gpu_solve(w, max_terms=40, tol=1e-4)
+        assert some_info == info[r0:r0 + 5]
+        assert np.array_equal(some, psi[r0:r0 + 5])
+        p.close()

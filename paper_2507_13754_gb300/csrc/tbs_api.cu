@@ -438,6 +438,7 @@ tbs_status enqueue_adjoint(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     TBS_CK(cudaMemsetAsync(p->Q, 0, sizeof(float2) * p->nrhs * nn, s));
     RowArgs ra = row_args(p);
     ra.src = p->G;
+    ra.num_sms = p->num_sms;  // the row variants are the forward pass's
     ColArgs ca = col_args(p);
     TBS_CK(timed_row(p, ROW_SRC, ra, s));  // X = FFT_x(ubar_{T-1} = g)
     ra.pdl = 1;  // the reverse steps' row passes follow their column passes programmatically
@@ -497,6 +498,7 @@ tbs_status enqueue_adjoint_ckpt(tbs_plan_s *p, cudaStream_t s, int tmax) {
     TBS_CK(cudaMemsetAsync(p->Q, 0, sizeof(float2) * slot, s));
     RowArgs ra = row_args(p);
     ra.src = p->G;
+    ra.num_sms = p->num_sms;  // the row variants are the forward pass's
     ColArgs ca = col_args(p);
     TBS_CK(timed_row(p, ROW_SRC, ra, s));  // X = FFT_x(ubar_{T-1} = g)
     ra.gate.mode = GATE_ADJ;

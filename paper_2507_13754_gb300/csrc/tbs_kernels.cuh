@@ -1064,9 +1064,9 @@ row_fwd_persistent_kernel(RowArgs a) {
 // slots of row_fwd_persistent_kernel, whose two half-row buffers
 // hold the Q and u_j rows here (both bulk-copied a row ahead, like W); g's row
 // is fetched into L2 meanwhile, V stays there.  The arithmetic per row is
-// exactly that of row_kernel<M, ROW_ADJ>.  One block per row loads W, Q, u_j,
-// g and V in turn between its transforms, each exposed to memory latency:
-// 302 us for 16 RHS at N = 1024, here 178 us.
+// exactly that of row_kernel<M, ROW_ADJ> (M < 512).  One block per row loaded W,
+// Q, u_j, g and V in turn between its transforms, each exposed to memory
+// latency: 302 us for 16 RHS at N = 1024, here 178 us.
 template <int M, int TH>
 __global__ void __launch_bounds__(RowPCfg<M, TH>::THREADS, 512 / TH)
 row_adj_persistent_kernel(RowArgs a) {
@@ -2270,17 +2270,17 @@ static cudaError_t row_launch_th(int nrhs, const RowArgs &b, cudaStream_t s) {
         if (b.n == M && b.num_sms > 0)
             return persistent_row<row_eps_persistent_kernel<M, KIND == ROW_EPSK, TH>, RowECfg<M, TH>>(nrhs, b, s);
     }
-    if constexpr ((KIND == ROW_FWD || KIND == ROW_ADJ) && M >= 512) {
-        if (b.num_sms > 0) {
-            if constexpr (KIND == ROW_FWD)
+    if constexpr (KIND == ROW_ADJ && M >= 512) {
+        return persistent_row<row_adj_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
+    } else {
+        if constexpr (KIND == ROW_FWD && M >= 512) {
+            if (b.num_sms > 0)
                 return b.n & 1 ? persistent_row<row_fwd_persistent_kernel<M, TH, true>, RowPCfg<M, TH>>(nrhs, b, s)
                                : persistent_row<row_fwd_persistent_kernel<M, TH, false>, RowPCfg<M, TH>>(nrhs, b, s);
-            else
-                return persistent_row<row_adj_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
         }
+        dim3 grid((b.n + C::RPB - 1) / C::RPB, nrhs);
+        return launch_k(row_kernel<M, KIND, TH>, grid, dim3(C::THREADS), C::SMEM, s, b.pdl != 0, b);
     }
-    dim3 grid((b.n + C::RPB - 1) / C::RPB, nrhs);
-    return launch_k(row_kernel<M, KIND, TH>, grid, dim3(C::THREADS), C::SMEM, s, b.pdl != 0, b);
 }
 
 template <int M, int KIND>
@@ -2548,7 +2548,7 @@ static cudaError_t row_attr() {
     };
     set(row_kernel<M, ROW_SRC, TH>, b);
     set(row_kernel<M, ROW_FWD, TH>, b);
-    set(row_kernel<M, ROW_ADJ, TH>, b);
+    if constexpr (M < 512) set(row_kernel<M, ROW_ADJ, TH>, b);
     set(row_kernel<M, ROW_VSRC, TH>, b);
     set(row_kernel<M, ROW_EPS, TH>, b);
     set(row_kernel<M, ROW_EPSK, TH>, b);

@@ -431,10 +431,12 @@ row_kernel(RowArgs a) {
     // shared memory: for even N (every row 16-byte aligned) by three bulk
     // copies per row, issued by the row's thread 0 and completing on two
     // barriers (bar[lr][0]: W, bar[lr][1]: psi and V) -- they bypass L1 and
-    // every thread waits on the barrier itself; for odd N by cp.async from
-    // every thread (W then needs a block barrier).
+    // every thread waits on the barrier itself; for odd N (M < 512: longer rows
+    // have the persistent pass) by cp.async from every thread (W then needs a
+    // block barrier).
     __shared__ __align__(8) uint64_t rbar[PREFETCH ? C::RPB : 1][2];
-    const bool bulk = PREFETCH && (n & 1) == 0;
+    constexpr bool CPASYNC = PREFETCH && M < 512;
+    const bool bulk = PREFETCH && (!CPASYNC || (n & 1) == 0);
     if (bulk && t == 0) {
         mbar_init(&rbar[lr][0], 1);
         mbar_init(&rbar[lr][1], 1);
@@ -458,7 +460,7 @@ row_kernel(RowArgs a) {
                 bulk_load(psi_s, a.psi + row_sp, (unsigned)(n * sizeof(float2)), &rbar[lr][1]);
                 bulk_load(v_s, a.V + (size_t)y * n, (unsigned)(n * sizeof(float2)), &rbar[lr][1]);
             }
-        } else {
+        } else if constexpr (CPASYNC) {
             if (valid) {
 #pragma unroll
                 for (int m = 0; m < E / 2; m++) cp_async16(line + 2 * (t + T * m), w + 2 * (t + T * m));
@@ -490,7 +492,7 @@ row_kernel(RowArgs a) {
                 mbar_wait_bounded(&rbar[lr][0], 0, a.wait_ns, a.err);
                 mbar_wait_bounded(&rbar[lr][1], 0, a.wait_ns, a.err);
             }
-        } else {
+        } else if constexpr (CPASYNC) {
             cp_async_wait<0>();
         }
         return;
@@ -523,7 +525,7 @@ row_kernel(RowArgs a) {
             // rows to their buffers: wait for W only
             if (bulk) {
                 if (valid) mbar_wait_bounded(&rbar[lr][0], 0, a.wait_ns, a.err);
-            } else {
+            } else if constexpr (CPASYNC) {
                 cp_async_wait<1>();
                 __syncthreads();
             }
@@ -555,7 +557,7 @@ row_kernel(RowArgs a) {
             // barrier; with cp.async a thread reads exactly the elements it copied
             if (bulk) {
                 if (valid) mbar_wait_bounded(&rbar[lr][1], 0, a.wait_ns, a.err);
-            } else {
+            } else if constexpr (CPASYNC) {
                 cp_async_wait<0>();
             }
             TBS_ROW_PHASE(3)
@@ -2274,7 +2276,7 @@ static cudaError_t row_launch_th(int nrhs, const RowArgs &b, cudaStream_t s) {
         return persistent_row<row_adj_persistent_kernel<M, TH>, RowPCfg<M, TH>>(nrhs, b, s);
     } else {
         if constexpr (KIND == ROW_FWD && M >= 512) {
-            if (b.num_sms > 0)
+            if (b.num_sms > 0 || (b.n & 1))  // an odd N has the persistent pass alone
                 return b.n & 1 ? persistent_row<row_fwd_persistent_kernel<M, TH, true>, RowPCfg<M, TH>>(nrhs, b, s)
                                : persistent_row<row_fwd_persistent_kernel<M, TH, false>, RowPCfg<M, TH>>(nrhs, b, s);
         }

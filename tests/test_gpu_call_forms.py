@@ -185,3 +185,29 @@ def test_reverse_sweep_is_the_same_for_both_row_variants(n):
     plan.close()
     assert np.abs(out[0][0]).max() > 0
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("n,max_terms", [(257, 30), (300, 20), (513, 12)])
+def test_checkpointed_sweep_of_persistent_passes(n, max_terms):
+    """M >= 512: the reverse pass bulk-copies the recomputed terms of a segment
+    (odd rows 8 bytes off a 16-byte boundary): bitwise the stored sweep, for RHS
+    with different term counts over several segments."""
+    import torch
+    from paper_2507_13754_gb300 import tbs, workloads as W
+    w = W.random_medium(n, seed=75, n_rhs=3)
+    w.src_amp[1] *= 0.5
+    w.src_amp[2] = 0
+    rng = np.random.default_rng(175)
+    g = (rng.standard_normal((3, n, n)) + 1j * rng.standard_normal((3, n, n))).astype(np.complex64)
+    out = []
+    for ck in (False, True):
+        psi, info, plan = gpu_solve(w, keep_terms=True, checkpoint=ck, max_terms=max_terms, tol=1e-12)
+        gc = torch.empty((n, n), dtype=torch.float32, device="cuda")
+        ga = torch.empty((n, n), dtype=torch.float32, device="cuda")
+        plan.solve_adjoint(torch.from_numpy(g).cuda(), gc, ga)
+        out.append((info, psi, gc.cpu().numpy(), ga.cpu().numpy()))
+        plan.close()
+    (i0, p0, c0, a0), (i1, p1, c1, a1) = out
+    assert i0 == i1 and i0[2]["terms"] == 1 and max(i["terms"] for i in i0) > 8
+    assert np.abs(c0).max() > 0 and np.array_equal(p0, p1)
+    assert np.array_equal(c0, c1) and np.array_equal(a0, a1)

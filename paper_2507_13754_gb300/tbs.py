@@ -10,6 +10,7 @@ library is not built, importing the binding fails loudly.
 from __future__ import annotations
 
 import ctypes as C
+import itertools
 import os
 import struct
 
@@ -226,17 +227,29 @@ def tbs_apply_green_noalloc(n, ghat_ptr, f_ptr, out_ptr, conj_kernel=0, stream=0
         n, ghat_ptr, f_ptr, out_ptr, int(conj_kernel), stream))
 
 
-def tbs_synthesize(entries, n_rhs, x0, y0, sx, sy, nx, ny, t0, dt, n_t, out_ptr, stream=0):
-    """entries: [(field_ptr, n, dx, freq_hz, weight)]; out [n_rhs][ny][nx][n_t] complex64."""
-    # one pack of all records (a ctypes structure per entry costs a microsecond)
+def _synth_records(entries, number=None):
+    """The records of [(field_ptr, n, dx, freq_hz, weight)] by one pack (a ctypes
+    structure per entry costs a microsecond); entries that struct does not take
+    as they are go through the structure, numbers through `number` if given."""
     arr = (tbs_synth_freq * len(entries))()
     try:
-        struct.pack_into("@" + "Pi0dddd" * len(entries), arr, 0, *[v for e in entries for v in e])
-    except struct.error:  # numbers in other forms
-        for a, (ptr, n, dx, f, w) in zip(arr, entries):
-            a.field, a.n, a.dx, a.freq_hz, a.weight = ptr, n, float(dx), float(f), float(w)
-    _check("tbs_synthesize", load_library().tbs_synthesize(arr, len(entries), n_rhs, x0, y0, sx, sy, nx, ny,
-                                                            t0, dt, n_t, out_ptr, stream))
+        if set(map(len, entries)) == {5}:
+            struct.pack_into("@" + "Pi0dddd" * len(entries), arr, 0, *itertools.chain.from_iterable(entries))
+            return arr
+    except (struct.error, TypeError, OverflowError):
+        pass
+    if number is not None:
+        entries = [(e[0], e[1], *map(number, e[2:])) for e in entries]
+    return (tbs_synth_freq * len(entries))(*[tbs_synth_freq(*e) for e in entries])
+
+
+def tbs_synthesize(entries, n_rhs, x0, y0, sx, sy, nx, ny, t0, dt, n_t, out_ptr, stream=0):
+    """entries: [(field_ptr, n, dx, freq_hz, weight)]; out [n_rhs][ny][nx][n_t] complex64."""
+    _synthesize(_synth_records(entries), n_rhs, x0, y0, sx, sy, nx, ny, t0, dt, n_t, out_ptr, stream)
+
+
+def _synthesize(arr, *args):
+    _check("tbs_synthesize", load_library().tbs_synthesize(arr, len(arr), *args))
 
 
 def synthesize(fields, dxs, freqs_hz, weights, origin, step, counts, t0, dt, n_t, out=None, stream=None):
@@ -256,8 +269,8 @@ def synthesize(fields, dxs, freqs_hz, weights, origin, step, counts, t0, dt, n_t
     if out is None:
         out = torch.empty((n_rhs, ny, nx, n_t), dtype=torch.complex64, device="cuda")
     ptr = _dev_ptr(out, torch.complex64, (n_rhs, ny, nx, n_t), "out")
-    tbs_synthesize(entries, n_rhs, float(origin[0]), float(origin[1]), float(step[0]), float(step[1]), nx, ny,
-                   float(t0), float(dt), n_t, ptr, _stream(stream))
+    _synthesize(_synth_records(entries, float), n_rhs, float(origin[0]), float(origin[1]), float(step[0]),
+                float(step[1]), nx, ny, float(t0), float(dt), n_t, ptr, _stream(stream))
     return out
 
 

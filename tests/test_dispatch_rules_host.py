@@ -76,3 +76,33 @@ def test_reverse_loops_launch_few_empty_steps(tmp_path):
         else:
             assert lead == 0 and 3 <= body <= 4
             assert -(-(m - 1) // body) == -(-(m - 1) // 4)  # as few iterations as bodies of 4
+
+
+def test_synthesis_records_in_every_form():
+    """The packed records are those of one structure per entry, for entries
+    given in part, numbers of other types and refusals alike."""
+    if shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"):
+        pytest.skip("nvcc not available to build the library")
+    import ctypes
+    import numpy as np
+    from paper_2507_13754_gb300 import build, tbs
+    build.build()
+    f = tbs.tbs_synth_freq
+    ok = [(0x1000, 8, 1e-4, 1e6, 1.0), (ctypes.c_void_p(0x2000), 8, 1e-4, 1e6, 1.0), (None, 9, 1, 2, 3),
+          (0x3000, 2 ** 31 + 5, 0.5, -1e300, float("inf")), (0x4000, 8, np.float32(0.1), np.float64(3), True),
+          (0x5000, 8), (0x6000, 8, 1e-4), ()]
+    for entries in [[e] for e in ok] + [ok, ok[:1], []]:
+        want = (f * len(entries))(*[f(*e) for e in entries])
+        assert bytes(tbs._synth_records(entries)) == bytes(want)
+    bad = [(0x1000, 8, "1e-4", 1e6, 1.0), (0x1000, 8.0, 1e-4, 1e6, 1.0), (0x1000, 8, 1e-4, 1e6, 1.0, 2.0)]
+    for entries in [[e] for e in bad] + [[ok[0], bad[0]], [(0x1000, 8, 1e-4, 1e6), bad[2]]]:
+        with pytest.raises(TypeError):
+            [f(*e) for e in entries]
+        with pytest.raises(TypeError):
+            tbs._synth_records(entries)
+    # synthesize() converts its numbers: text too
+    text = tbs._synth_records([(0x1000, 8, "1e-4", "1e6", "0.5")], float)
+    assert bytes(text) == bytes((f * 1)(f(0x1000, 8, 1e-4, 1e6, 0.5)))
+    # short records reach the library's own checks (n_t = 0 is refused before any launch)
+    with pytest.raises(tbs.TbsError):
+        tbs.tbs_synthesize([(0x1000, 8)], 1, 0.0, 0.0, 1e-4, 1e-4, 1, 1, 0.0, 1e-8, 0, 0x2000)

@@ -392,12 +392,16 @@ tbs_status tbs_get_timing(tbs_plan_t plan, double *row_ms, int32_t *row_launches
  * more resident blocks per SM) and, for M >= 1024, the pipelined kernel
  * (one or two columns per thread, the latter also with the two columns
  * staggered); at M = 4096 the pipelined kernel with two columns per thread
- * comes first, at M = 2048 the compact one (two blocks per SM), at M = 512 and
- * 1024 the narrowed lockstep tiles.  At
+ * comes first, at M = 2048 the compact one (two columns per thread, two blocks
+ * per SM; it stands in place of the pipelined kernel with one column per
+ * thread), at M = 512 and 1024 the narrowed lockstep tiles.  M = 128 and 256 have
+ * one variant, narrowed where the plan has few right-hand sides.  At
  * M = 4096 the list also holds the two-column pipelined kernel with the FFT
- * split into four radix-8 stages instead of three radix-16 ones; periodic plans have the lockstep kernel with two and with
- * one column per thread and, for M >= 1024, the pipelined kernel with two
- * columns per thread (plain and staggered).  Variants with the same radix
+ * split into four radix-8 stages instead of three radix-16 ones.  Periodic
+ * plans have two lockstep passes, with two columns per thread (the compact
+ * kernel at M = 1024 and 2048, a narrow tile at M = 256 .. 1024 for few
+ * right-hand sides) and with one, and, for M >= 1024, the pipelined kernel with
+ * two columns per thread (plain and staggered).  Variants with the same radix
  * split give bitwise the same result; the radix-8 split rounds differently
  * (agreement to FP32 rounding, the same parity with the exact operator).
  * tbs_col_variant_name describes variant v (v < 0: the active one) in a
@@ -419,8 +423,10 @@ tbs_status tbs_autotune(tbs_plan_t plan, int32_t reps, double *times_ms, int32_t
  * each taking rows in a fixed stride and bulk-copying the next row's inputs
  * while it transforms the current one), variant 1 launches one block per
  * row.  The persistent variant exists for M >= 512; an odd N has it alone,
- * and plans with M < 512 have variant 0 only, one block per row.  Both give bitwise the same result.  tbs_row_variants,
- * tbs_row_variant_name and tbs_set_row_variant work as their column-pass
+ * and plans with M < 512 have variant 0 only, one block per row.  Both give
+ * bitwise the same field (the records agree to FP32 rounding of the norms).
+ * The reverse sweep of tbs_solve_adjoint does not depend on the variant.
+ * tbs_row_variants, tbs_row_variant_name and tbs_set_row_variant work as their column-pass
  * counterparts.  tbs_autotune_rows times each variant (`reps` launches after
  * a warm-up, on `stream`, synchronously) at a steady-state term on the
  * plan's current medium and intermediates, activates the fastest and

@@ -1220,7 +1220,7 @@ int32_t tbs_col_variants(tbs_plan_t p) { return p ? col_variants(p->M, p->period
 
 const char *tbs_col_variant_name(tbs_plan_t p, int32_t variant) {
     if (!p) return nullptr;
-    return col_variant_name(p->M, p->periodic, variant < 0 ? p->col_variant : variant);
+    return col_variant_name(p->M, p->nrhs, p->periodic, variant < 0 ? p->col_variant : variant);
 }
 
 tbs_status tbs_set_col_variant(tbs_plan_t p, int32_t variant) {

@@ -276,15 +276,18 @@ cudaError_t launch_row(int kind, int M, int nrhs, const RowArgs &a, cudaStream_t
 
 int col_variants(int M, bool periodic) { return periodic ? col_periodic_variant_count(M) : col_variant_count(M); }
 
-const char *col_variant_name(int M, bool periodic, int variant) {
+const char *col_variant_name(int M, int nrhs, bool periodic, int variant) {
     if (variant < 0 || variant >= col_variants(M, periodic)) return nullptr;
     if (periodic) {
+        // two columns per thread in lockstep: col_kernel, its narrow tile for few
+        // RHS, or the compact kernel
         if (col_variants(M, true) == 1) return "periodic, lockstep, 1 column/thread";
         static const char *names[4] = {"periodic, lockstep, 2 columns/thread", "periodic, lockstep, 1 column/thread",
                                        "periodic, pipelined, 2 columns/thread",
                                        "periodic, pipelined, 2 columns/thread, staggered"};
         return names[variant];
     }
+    if (col_narrow(M, nrhs, false)) return "tile narrowed for few right-hand sides (lockstep)";
     switch (col_variant_kind(M, variant)) {
     case COL_S0: return "tile S0 (lockstep, default width)";
     case COL_S1: return "tile S1 (lockstep, width/2)";

@@ -2421,10 +2421,12 @@ static cudaError_t with_col_variant_per(int variant, int nrhs, bool ks, F f) {
     // fastest first as measured on GB300: at M = 1024 and 2048 the compact
     // kernel, else two columns per thread of col_kernel, then one (the only
     // shape below M = 32)
-    if constexpr (col_periodic_compact(M))
-        if (variant == 0) return ks ? f(ColCompact<M, 8192 / M, 2>{}) : f(ColCompact<M, 8192 / M, 1>{});
     if constexpr (col_periodic_variant_count(M) > 1) {
-        if (variant == 0) return ks ? f(ColCfgPK2<M>{}) : f(ColCfgP2<M>{});
+        if constexpr (col_periodic_compact(M)) {
+            if (variant == 0) return ks ? f(ColCompact<M, 8192 / M, 2>{}) : f(ColCompact<M, 8192 / M, 1>{});
+        } else {
+            if (variant == 0) return ks ? f(ColCfgPK2<M>{}) : f(ColCfgP2<M>{});
+        }
         if (variant == 1) return ks ? f(ColCfgPK<M>{}) : f(ColCfgP<M>{});
     } else {
         if (variant == 0) return ks ? f(ColCfgPK<M>{}) : f(ColCfgP<M>{});

@@ -211,3 +211,13 @@ def test_checkpointed_sweep_of_persistent_passes(n, max_terms):
     assert i0 == i1 and i0[2]["terms"] == 1 and max(i["terms"] for i in i0) > 8
     assert np.abs(c0).max() > 0 and np.array_equal(p0, p1)
     assert np.array_equal(c0, c1) and np.array_equal(a0, a1)
+
+
+@pytest.mark.parametrize("n,n_rhs,narrow", [(64, 1, True), (64, 4, True), (64, 5, False), (128, 2, True),
+                                            (128, 3, False), (32, 1, False)])
+def test_variant_names_tell_narrowed_tiles(n, n_rhs, narrow):
+    from paper_2507_13754_gb300 import tbs
+    p = tbs.Plan(n, 1e-4, 1e6, 1500.0, n_rhs=n_rhs)
+    name = tbs.tbs_col_variant_name(p.handle)
+    assert ("narrowed" in name) == narrow and ("default width" in name) == (not narrow)
+    p.close()

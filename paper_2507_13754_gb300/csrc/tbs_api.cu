@@ -347,9 +347,12 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     // 11.1 / 15.5 / 36.7 us, of the periodic 4096^2 grid 241 -> 232 us
     const bool fused = p->M >= 128;
     const bool early = early_columns(p);
-    // The smallest passes leave room for the row pass's blocks beside them: a
-    // term at N = 256 14.2 -> 12.5 us (at N = 512 16.2 -> 17.0 us: not there).
-    const bool beside = (size_t)p->nrhs * p->n * p->M <= (size_t)256 * 512;
+    // The smallest passes leave room for the row pass's blocks beside them: 24
+    // terms at N = 32 (8 RHS) / 64 (2 RHS) / 100 289 / 231 / 231 -> 279 / 210 / 220 us.
+    // Above, the row blocks' early start takes more from the column pass than it
+    // saves: N = 128 / 200 / 256 213 / 289 / 250 -> 218 / 299 / 255 us, 4 RHS at N = 128
+    // 247 -> 264 us, N = 300 334 -> 363 us.
+    const bool beside = (size_t)p->nrhs * p->n * p->M < (size_t)32 * 1024;
     // which rows of V are one repeated value and which source rows are zero
     // (the medium and sources may change between solves of a plan)
     if (rk == ROW_EPS) TBS_CK(launch_row_flags(p->n, p->nrhs, p->V, p->S, p->vflag, p->sflag, s));
@@ -412,8 +415,10 @@ bool kernel_may_use(const tbs_plan_s *p, const void *ptr, size_t align) {
 }
 
 // The outputs of the solve enqueued on s: psi and the records to the caller's
-// buffers.  Small fields travel in the kernel that writes the records (a
-// 256^2 solve is three launches shorter); larger ones by a device copy.
+// buffers.  Fields of up to 4 MB travel in the kernel that writes the records
+// (4 terms at N = 256 / 512 / 700 66.8 / 82.8 / 162.4 -> 62.8 / 77.8 / 153.8 us); larger
+// ones by a device copy (the kernel would save as many microseconds, below 3%:
+// 1024^2 169 -> 165, 2048^2 536 -> 532 us).
 tbs_status enqueue_outputs(tbs_plan_s *p, float *psi, tbs_solve_info *info, bool device_info, cudaStream_t s) {
     const size_t count = (size_t)p->nrhs * p->n * p->n;
     const bool direct = device_info && kernel_may_use(p, info, 8);

@@ -2034,7 +2034,8 @@ col_pipe_kernel(ColArgs a, const __grid_constant__ CUtensorMap tmx, const __grid
 // (27.8 in lockstep), 24.6 us for 4 x 1024^2 (28.8).  At M = 4096 the lines
 // leave two columns per tile and nothing is gained (71.3 against 71.7 us
 // padded, 125 against 98 us periodic); tiles of four columns with one block of
-// 512 threads: 72 and 123 us.
+// 512 threads: 72 and 123 us.  The plain periodic instances spill 20 bytes at the
+// 128 registers that two blocks of 256 threads leave; the times above include it.
 template <int M, int TC_, int PER_ = 0>
 struct ColCompact : ColShape<M, TC_, 2, 2, PER_> {
     using B_ = ColShape<M, TC_, 2, 2, PER_>;
@@ -2257,9 +2258,10 @@ static cudaError_t persistent_row(int nrhs, const RowArgs &b, cudaStream_t s) {
 }
 
 // Blocks of 64 threads instead of 256 where the latter would not give every SM
-// one (152 SMs).  With the column tiles and launches of small problems a term
-// at N = 256 went from 15.5 to 12.5 us, at N = 64 from 11.1 to 10.3 us; at
-// M = 1024 (N = 512) nothing was gained.
+// one (GB300 has 152; a constant, since RowArgs::num_sms is 0 in some launches).
+// With the column tiles and launches of small problems a term at N = 256 went
+// from 15.5 to 12.5 us, at N = 64 from 11.1 to 10.3 us; at M = 1024 (N = 512)
+// nothing was gained.
 __host__ __device__ constexpr bool row_has_small(int M) { return M <= 512; }
 static inline bool row_small(int M, int nrhs, int n) {
     return row_has_small(M) && (size_t)nrhs * n * (M / 16) <= 152 * 256;

@@ -3,8 +3,8 @@
 ``tune(plan)`` asks the library to time every compiled column-pass variant
 (tile width, columns per thread, pipelined or lockstep staging) on the plan's
 own buffers (tbs_autotune) and every steady-state row-pass variant
-(persistent or one block per row; tbs_autotune_rows), and keeps the fastest
-of each.  Results are cached per (GPU, kernel sources, M, n_rhs, grid kind)
+(the forward pass: persistent or one block per row; tbs_autotune_rows), and
+keeps the fastest of each.  Results are cached per (GPU, kernel sources, M, n_rhs, grid kind)
 so later plans reuse the choice with tbs_set_col_variant and
 tbs_set_row_variant instead of timing again, and a rebuilt library with
 changed kernels times afresh.
@@ -30,8 +30,8 @@ def _gpu_name():
 
 
 def _key(plan):
-    # the row shapes available depend on N as well as M (odd N has no
-    # persistent row pass), so their count is part of the key
+    # the row shapes available depend on N as well as M (an odd N has one of
+    # them alone), so their count is part of the key
     return "%s|src=%s|M=%d|nrhs=%d|%s|row_shapes=%d" % (_gpu_name(), build.source_hash(), plan.m, plan.n_rhs,
                                                         "periodic" if plan.periodic else "padded",
                                                         tbs.tbs_row_variants(plan.handle))

@@ -360,7 +360,6 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
         // Each kernel reads its RHS's term index from the RHS state and returns
         // at once for an RHS that has stopped.  The stop test at the end of the
         // lead and of each body sets the loop's condition.
-        ca.gate.mode = ra.gate.mode = GATE_FWD;
         ra.term = sa.term = -1;
         auto terms = [&](cudaStream_t b, int count, const cudaGraphConditionalHandle *h) {
             cudaError_t e = cudaSuccess;

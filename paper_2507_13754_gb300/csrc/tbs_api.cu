@@ -96,7 +96,7 @@ struct tbs_plan_s {
     double2 *part = nullptr, *l1 = nullptr;
     RhsState *state = nullptr;
     double *norms = nullptr;
-    int *err = nullptr;              // device words: [0] error of bounded waits, [1..2] graph-loop control
+    int *err = nullptr;              // device words (ERR_WORDS)
     ColMaps cmaps[MAX_COL_VARIANTS];                // X and W tensor maps of the column pass, per variant
     int col_variant = 0;             // active column-pass tile shape
     int row_variant = 0;             // steady-state row pass: 0 persistent, 1 one block per row
@@ -330,6 +330,7 @@ tbs_status enqueue_solve(tbs_plan_s *p, cudaStream_t s, bool graph_loop) {
     sa.div_grace = p->d.div_grace;
     sa.div_window = p->d.div_window;
     sa.div_factor = p->d.div_factor;
+    sa.stopped = p->err + 4;
     sa.sums = stop_sums(p->M);
     sa.loop_ctl = nullptr;
     sa.loop = 0;
@@ -617,7 +618,7 @@ static PlanLayout plan_layout(const tbs_plan_desc *d) {
     sz[B_STATE] = r * sizeof(RhsState);
     sz[B_NORMS] = r * T * sizeof(double);
     sz[B_INFO] = r * sizeof(tbs_solve_info);
-    sz[B_ERR] = 4 * sizeof(int);
+    sz[B_ERR] = ERR_WORDS * sizeof(int);
     const bool ckpt = keep && (d->flags & TBS_FLAG_CHECKPOINT_TERMS);
     const size_t K = ckpt ? ckpt_every(d->max_terms) : 0, ncp = ckpt ? (T + K - 1) / K : 0;
     sz[B_U] = keep ? (ckpt ? ncp : T) * r * nn * sizeof(float2) : 0;
@@ -790,7 +791,7 @@ static tbs_status plan_create(const tbs_plan_desc *d, void *workspace, size_t wo
         (!p->periodic || (e = cudaMemcpyAsync(p->abl, abl_host.data(), sizeof(float) * p->M,
                                               cudaMemcpyHostToDevice, s)) == cudaSuccess) &&
         (e = cudaMemsetAsync(p->state, 0, r * sizeof(RhsState), s)) == cudaSuccess &&
-        (e = cudaMemsetAsync(p->err, 0, 4 * sizeof(int), s)) == cudaSuccess &&
+        (e = cudaMemsetAsync(p->err, 0, ERR_WORDS * sizeof(int), s)) == cudaSuccess &&
         (e = cudaMemsetAsync(p->psi, 0, r * nn * sizeof(float2), s)) == cudaSuccess) {
         e = cudaStreamSynchronize(s);
     }

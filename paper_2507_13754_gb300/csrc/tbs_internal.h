@@ -90,6 +90,10 @@ struct Gate {
     int back;            // less this many (negative: no step)
 };
 
+// A plan's device words: [0] error of bounded waits, [1..2] graph-loop control,
+// [3] the reverse sweep's step, [4] RHS stopped in this solve.
+constexpr int ERR_WORDS = 5;
+
 // Row-pass variants.
 enum RowKind {
     ROW_SRC = 0,       // y = src (spatial)              -> forward FFT -> X
@@ -127,6 +131,7 @@ struct StopArgs {
     int div_grace;
     int div_window;
     double div_factor;
+    int *stopped;       // counts the RHS that have stopped in this solve
     int sums;           // stop_sums(M)
     int pdl;            // launch as a programmatic dependent of the previous kernel
 };
@@ -168,7 +173,7 @@ struct RowArgs {
     // them (the RHS states; the error words), or none
     void *clear;
     int clear_words;
-    int *clear_err;     // 4 words, or null
+    int *clear_err;     // ERR_WORDS words, or null
 };
 
 struct ColArgs {

@@ -221,3 +221,38 @@ def test_variant_names_tell_narrowed_tiles(n, n_rhs, narrow):
     name = tbs.tbs_col_variant_name(p.handle)
     assert ("narrowed" in name) == narrow and ("default width" in name) == (not narrow)
     p.close()
+
+
+def test_a_series_that_ends_costs_no_column_pass():
+    """The column pass under way when the last series ends is broken off: two
+    terms to a residual take less than three quarters of a column pass more than
+    two terms that nothing follows (least of many runs)."""
+    import torch
+    from paper_2507_13754_gb300 import workloads as W
+
+    def least(plan):
+        psi, _ = plan.solve()
+        info = torch.empty(64 * plan.n_rhs, dtype=torch.uint8, device="cuda")
+        ms = []
+        for _ in range(40):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            plan.solve(psi=psi, info=info, sync=False)
+            b.record()
+            b.synchronize()
+            ms.append(a.elapsed_time(b))
+        return min(ms)
+
+    w = W.random_medium(1024, seed=76, n_rhs=8)
+    w.alpha *= np.float32(0.05)  # weak enough for the second term to be the smaller one
+    w.c[:] = 1500 + (w.c - 1500) * np.float32(0.1)
+    _, info, two = gpu_solve(w, max_terms=2, tol=0.0)
+    _, to_tol, series = gpu_solve(w, max_terms=64, tol=max(i["residual"] for i in info) * (1 + 1e-6))
+    assert [i["terms"] for i in to_tol] == [2] * 8
+    extra = least(series) - least(two)
+    two.set_timing()
+    two.solve()
+    _, _, col_ms, cols = two.timing()
+    assert extra < 0.75 * col_ms / cols, (extra, col_ms / cols)
+    two.close()
+    series.close()

@@ -741,10 +741,15 @@ def run_ours(args, rank, world, local_rank):
     units = n * n * sum(terms)
     t_max, units_all = aggregate_ranks(t_total, units, world, dev)
     value = units_all / t_max
-    # medium, deposit, row(src), (col, row, stop) per term slot, info: the
-    # graph's term loop runs bodies of four terms until every RHS has
-    # stopped (one RHS here), so max(terms) rounds up to a multiple of four
-    launches = sum(2 + 1 + 3 * (4 * -(-t // 4)) + 1 for t in terms)
+    # medium, deposit, row(src), finish; (col, row) per term slot and a stop test
+    # at the end of each part: the graph holds 4 terms ahead of its loop, whose
+    # bodies are of 8 (max_terms 64); from the host, max_terms slots and one test
+    def step_launches(t):
+        if args.no_graph:
+            return 4 + 2 * w.max_terms + 1
+        bodies = -(-max(t - 4, 0) // 8)
+        return 4 + 2 * (4 + 8 * bodies) + 1 + bodies
+    launches = sum(step_launches(t) for t in terms)
 
     if args.kernel_only:
         if rank == 0:

@@ -38,10 +38,10 @@ struct RhsState {
 // 14 us (N >= 700) per iteration beyond its launches, also when it is not
 // entered, a term's launches after the stop 3 to 7 us.
 //  * to a residual: 4 terms, then equal bodies of at most 8.  With 8-term
-//    bodies alone a series of one term paid for 8: 111 -> 88 us at N = 700,
-//    122 -> 99 us at N = 1024 (101 us with bodies of 4).  Longer series end in
-//    another place of a body: at N = 700, 8 / 12 / 16 / 20 terms 286 / 455 / 549
-//    / 719 -> 322 / 415 / 584 / 677 us (338 / 491 / 644 / 795 us with bodies of 4).
+//    bodies alone a series of one term paid for 8: 111 -> 86 us at N = 700,
+//    122 -> 103 us at N = 1024 (97 and 101 us with bodies of 4).  Longer series end
+//    in another place of a body: at N = 700, 8 / 12 / 16 / 20 terms 286 / 455 / 549
+//    / 719 -> 325 / 418 / 587 / 679 us (338 / 491 / 644 / 795 us with bodies of 4).
 //  * a fixed number of terms: the WHILE alone, with the body (at most 16) of
 //    the least cost at 7 us an iteration and 4 us an empty term.
 struct TermLoop {
